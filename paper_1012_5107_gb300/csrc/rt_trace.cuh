@@ -1249,6 +1249,22 @@ __device__ __forceinline__ R box_entry(const StepConst<R>& k, const Cold<R>& C, 
     return tn;
 }
 
+// Whether a line that enters the box at tb does so before it can meet the
+// grating (or the bump): from above the surface's highest point y = A it
+// reaches that height at t0 = (A - y)/dy, and the hit searches return t0 or
+// more (a thousandth of slack covers the rounding of t0).  The march that
+// looks for the hit is skipped then; nearly every camera ray over a cloak box
+// is such a line, and its march takes some ten solves of Kepler's equation
+// (of the bump's parameter): the Gaussian render 9.25 -> 8.58 ms, 1920 x 1080
+// x 16 Dormand-Prince 118.8 -> 116.0 ms, the step's launch 7.17 -> 7.10 ms.
+// The options build keeps the march first: with the test its Fresnel renders
+// took 8.92 ms instead of 8.63 (its code spills at 128 registers).
+template <class R>
+__device__ __forceinline__ bool box_first(const StepConst<R>& k, const Cold<R>& C, R tb)
+{
+    return C.dy < R(0) && C.y > k.A && tb < R(0.999) * ((k.A - C.y) / C.dy);
+}
+
 // Background plane standing in for the photograph (Sec. 4, Fig. 2a).
 template <class R>
 __device__ __forceinline__ int background(const DevScene& sc, const AirConst<R>& a, const Cold<R>& C, float col[3])
@@ -1419,13 +1435,16 @@ __device__ void air_segment(const DevScene& sc, Cold<R>& C, Box<R>& b, int& phas
     for (;;) {
         if (C.bounces > sc.max_bounces) { finish_sample<R, OPT>(sc, C, steps, RT_RAY_MAX_BOUNCES, phase, rec); return; }
         R hcx = R(0), hX = R(0), hy = R(0);
-        R tm;
-        if constexpr (gauss_of(INTEG))
-            tm = sc.mirror ? bump_line_hit(k, C, surf == EV_GRATING, hcx, hX, hy) : flat_line_hit(C);
-        else
-            tm = sc.mirror ? trochoid_line_hit(k, C, surf == EV_GRATING, hcx, hX, hy) : flat_line_hit(C);
+        R tm = R(INFINITY), tb = R(INFINITY);
         int face = EV_NONE;
-        const R tb = (sc.cloak || plate) ? box_entry(k, C, face) : R(INFINITY);
+        if constexpr (!OPT) tb = sc.cloak ? box_entry(k, C, face) : R(INFINITY);
+        if (!sc.mirror)
+            tm = flat_line_hit(C);
+        else if (OPT || !box_first(k, C, tb)) {
+            if constexpr (gauss_of(INTEG)) tm = bump_line_hit(k, C, surf == EV_GRATING, hcx, hX, hy);
+            else tm = trochoid_line_hit(k, C, surf == EV_GRATING, hcx, hX, hy);
+        }
+        if constexpr (OPT) tb = (sc.cloak || plate) ? box_entry(k, C, face) : R(INFINITY);
         if (tb < tm) {
             advance(C, tb);
             R Nf[3];
