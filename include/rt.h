@@ -69,7 +69,9 @@ extern "C" {
                                  time t (state r, v with |v| = c0/n), fixed
                                  step h in t; wavefront loop only              */
 #define RT_FP32 0             /* single precision bulk arithmetic              */
-#define RT_FP64 1             /* double precision throughout                   */
+#define RT_FP64 1             /* double precision throughout (rt_split.cuh:
+                                 partly as sums of two and three floats, with
+                                 no more rounding)                             */
 
 /* per-ray status */
 #define RT_RAY_OK 0           /* reached the background                        */

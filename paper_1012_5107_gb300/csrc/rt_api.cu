@@ -220,6 +220,21 @@ static void build_dev(const rt_scene_desc* d, DevScene* s)
         s->cf.far24 = reach > 4.0 * (double)Mth<float>::kPredTol ? 1.0f : 0.0f;
         s->cd.far24 = reach > 4.0 * Mth<double>::kPredTol ? 1.0 : 0.0;
     }
+    // The split double precision step (rt_split.cuh): plain grating cloaks, RK4
+    // in tau, within the bounds its series are cut for -- kA <= 0.3 and a
+    // step's |s| = k h |p| <= 1/16 (the benchmark's h = Lambda/200 has 0.042
+    // at kA = 0.25) -- and with |W0| >= kA exp(-50) in the box, where its
+    // FP32 parts keep their relative precision.
+    {
+        const double pmax = 1.001 / (1.0 - s->kA);
+        s->sp.kh = kTwoPi * s->h;
+        s->sp.ikh = 1.0 / s->sp.kh;
+        const double kappa = s->sp.kh * s->sp.kh * (s->cd.fk * (1.0 / kTwoPi));
+        s->sp.kappa.h = (float)kappa;
+        s->sp.kappa.l = (float)(kappa - (double)s->sp.kappa.h);
+        s->sp.ok = d->cloak && d->mirror == RT_MIRROR_TROCHOID && d->flags == 0 && d->integrator == RT_RK4 &&
+                   s->kA <= 0.3 && s->sp.kh * pmax <= 1.0 / 16.0 && s->sp.kh >= 1e-6 && kTwoPi * s->ytop <= 50.0;
+    }
     s->cd.ybot = ((d->flags & RT_FLAG_PLATE) || d->mirror == RT_MIRROR_GAUSS) ? 0.0 : -s->A;
     s->cf.ybot = (float)s->cd.ybot;
     // Gaussian bump: width, 1/width, k h, h/width, the Newton stop on W and
@@ -317,10 +332,10 @@ int rt_create_scene(const rt_scene_desc* desc, rt_scene** out)
     build_dev(desc, &s->dev);
     int bps = 0;
     s->variant = kDefaultVariant;
-    s->min_active = default_min_active(desc->precision, render_mode(*desc));
+    s->min_active = default_min_active(desc->precision, wave_mode(desc->precision, render_mode(*desc), s->dev));
     s->wait = WaitLimit{kDefaultWaitSpin, 0};
     cudaError_t e = desc->mirror == RT_MIRROR_GAUSS ? gauss_upload() : cudaSuccess;
-    if (e == cudaSuccess) e = render_occupancy(desc->precision, render_mode(*desc), s->variant, desc->flags != 0, &bps);
+    if (e == cudaSuccess) e = render_occupancy(desc->precision, wave_mode(desc->precision, render_mode(*desc), s->dev), s->variant, desc->flags != 0, &bps);
     int nsm = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     s->nsm = nsm;
@@ -476,7 +491,7 @@ int rt_scene_autotune(rt_scene* s, float* d_rgb, int32_t trials, void* stream, i
     char key[160];
     snprintf(key, sizeof key, "scene/p%d/i%d/c%d/m%d/f%d/log2n%d", d.precision, d.integrator, d.cloak, d.mirror, d.flags,
              (int)floor(log2(samples > 1.0 ? samples : 1.0)));
-    int v = kDefaultVariant, m = default_min_active(d.precision, render_mode(d));
+    int v = kDefaultVariant, m = default_min_active(d.precision, wave_mode(d.precision, render_mode(d), s->dev));
     if (!tune_lookup(key, &v, &m)) {
         const int cand[] = {12, 16, 20, 24, 28};
         cudaStream_t st = (cudaStream_t)stream;
@@ -529,7 +544,8 @@ int rt_scene_set_launch(rt_scene* s, int32_t variant, int32_t min_active)
     RT_REQ(min_active == 0 || (min_active >= 1 && min_active <= 32), "min_active must be 0 (keep) or 1..32");
     if (variant >= 0 && variant != s->variant) {
         int bps = 0;
-        RT_CK(render_occupancy(s->desc.precision, render_mode(s->desc), variant, s->desc.flags != 0, &bps));
+        RT_CK(render_occupancy(s->desc.precision, wave_mode(s->desc.precision, render_mode(s->desc), s->dev), variant,
+                               s->desc.flags != 0, &bps));
         RT_REQ(bps > 0, "variant %d does not fit on this device", variant);
         s->variant = variant;
         s->grid = bps * s->nsm;

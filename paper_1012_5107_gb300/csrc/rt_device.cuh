@@ -10,6 +10,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "rt_split.cuh"
+
 namespace grt {
 
 constexpr double kPi = 3.14159265358979323846;
@@ -52,6 +54,14 @@ struct AirConst {
     R inv_cell, inv_texel;
 };
 
+// Constants of the split double precision step (rt_split.cuh): kappa = k h^2 fk,
+// k h and its inverse; ok: the scene is within the step's bounds.
+struct SplitConst {
+    F2 kappa;
+    double kh, ikh;
+    int ok;
+};
+
 struct DevScene {
     StepConst<float> cf;
     StepConst<double> cd;
@@ -80,6 +90,7 @@ struct DevScene {
     int flags;                              // RT_FLAG_*
     double idx_scale;                       // index scale inside the cloak (1 + kA when referenced)
     double plate_n;                         // index of the dielectric plate (1 + kA)
+    SplitConst sp;
 };
 
 // ------------------------------------------------------------------------

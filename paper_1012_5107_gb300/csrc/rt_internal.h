@@ -23,10 +23,13 @@ constexpr int kDefaultVariant = kVariantWave;
 // at 28, 7.87 at 30); the FP32 time form and Gaussian medium at 28 (time form
 // 9.21 ms, 9.35 at 24, 9.47 at 30; Gaussian 9.39 / 9.49 ms at 28 / 24); the
 // FP64 loops, bound by the FP64 pipe, with full warps only (FP64 cloaked
-// render 590 ms at 32, 595 at 30, 605 at 28, 623 at 24).
+// render 590 ms at 32, 595 at 30, 605 at 28, 623 at 24); the split double
+// precision step at 28 (the same render 39.2 ms, 39.0 at 30, 39.3 at 24, 39.8
+// at 16; 64 x 64 x 1 is 3 % faster with fewer).
 constexpr int kMinActive = 28;
 constexpr int kMinActiveRK4F32 = 24;
 constexpr int kMinActiveF64 = 32;
+constexpr int kMinActiveSplit = 28;
 // Dormand-Prince steps are longer: a task holding fewer rays is still worth
 // running (1920 x 1080 x 16 with one block of 384 threads per SM, E = 8 / 32:
 // 133.0 / 214.8 ms at 8, 135.1 / 221.5 ms at 16; 2 to 10 within 1 %)
@@ -36,6 +39,7 @@ constexpr int kMinActiveDP45 = 8;
 inline int default_min_active(int precision, int mode)
 {
     if ((mode & 7) == RT_DP45) return kMinActiveDP45;
+    if (mode & 16) return kMinActiveSplit;
     if (precision == RT_FP64) return kMinActiveF64;
     if (mode == RT_RK4) return kMinActiveRK4F32;
     return kMinActive;
@@ -43,10 +47,18 @@ inline int default_min_active(int precision, int mode)
 constexpr int kMaxWindows = 16;
 // Render mode: the integrator (RT_RK4, RT_DP45, RT_RK4T), with kModeGauss set
 // for scenes of the Gaussian bump, whose box holds the Gaussian map's medium.
+// kModeSplit: FP64 RK4 in the grating cloak with the step of rt_split.cuh, for
+// scenes within its bounds (SplitConst::ok); wavefront loop only.
 constexpr int kModeGauss = 8;
+constexpr int kModeSplit = 16;
 inline int render_mode(const rt_scene_desc& d)
 {
     return d.integrator | (d.mirror == RT_MIRROR_GAUSS ? kModeGauss : 0);
+}
+// The mode of the wavefront loop a scene is rendered with.
+inline int wave_mode(int precision, int mode, const DevScene& sc)
+{
+    return precision == RT_FP64 && mode == RT_RK4 && sc.sp.ok ? mode | kModeSplit : mode;
 }
 // Coefficients of the Faddeeva series of the Gaussian cloak, uploaded once
 // per device before its first Gaussian scene.

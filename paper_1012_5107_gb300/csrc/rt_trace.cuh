@@ -50,6 +50,9 @@ namespace grt {
 // conformal cloak (rt_gauss.cuh) in place of the grating cloak of Eq. 1.
 __host__ __device__ constexpr int integ_of(int mode) { return mode & 7; }
 __host__ __device__ constexpr bool gauss_of(int mode) { return (mode & kModeGauss) != 0; }
+// kModeSplit: the integration loop steps a SplitBox (rt_split.cuh) instead of
+// a Box<double>; the service code is the FP64 path's.
+__host__ __device__ constexpr bool split_of(int mode) { return (mode & kModeSplit) != 0; }
 
 enum : int { PH_IDLE = 0, PH_AIR = 1, PH_BOX = 2, PH_DONE = 3, PH_EXIT = 4, PH_EVENT = 5, PH_GUARD = 6 };
 enum : int { EV_NONE = -1, EV_GRATING = 0, EV_TOP = 1, EV_XP = 2, EV_XM = 3, EV_ZP = 4, EV_ZM = 5, EV_COUNT = 6 };
@@ -292,6 +295,18 @@ __device__ __forceinline__ bool w0_continue(const StepConst<R>& k, R X, R y, R d
     if constexpr (sizeof(R) == 8) w0_predict3(wr, wi, rr, ri, dx, dy);
     w0_eval(k, X, y, wr, wi, rr, ri, st);
     return true;
+}
+
+// A cold start of the FP64 solve: W0 to FP32, from which one FP64 Newton step
+// (a library exponential and sine/cosine each) is left of five.
+__device__ __forceinline__ void w0_seed(const StepConst<float>& k, double X, double y, double& wr, double& wi)
+{
+    float fr = 0.0f, fi = 0.0f, rr, ri;
+    w0_solve(k.kA, k.w0tol, (float)X, (float)y, fr, fi, rr, ri);
+    if (isfinite(fr) && isfinite(fi)) {
+        wr = (double)fr;
+        wi = (double)fi;
+    }
 }
 
 // ------------------------------------------------------------------------
@@ -819,12 +834,69 @@ __device__ __forceinline__ void dp45_step(const StepConst<R>& k, const Box<R>& s
         dp45_step_table<R, INTEG>(k, s, h, o, e, st);
 }
 
+// The split double precision step (rt_split.cuh) between the service's FP64
+// states: W0 is carried by factors, so it must be good relative to itself.  A
+// cold start at |W0| < 1e-8 stops within 1e-8 of it (w0_converged is
+// absolute), so a small W0 takes one more Newton step before it is carried.
+__device__ __forceinline__ void split_polish(double kA, double X, double y, double& wr, double& wi)
+{
+    if (wr * wr + wi * wi < 1e-14) {
+        double rr, ri, dr, di;
+        newton_w0(kA, X, y, wr, wi, rr, ri, dr, di);
+    }
+}
+
+__device__ __forceinline__ void split_state(const Box<double>& b, double kh, F2 kappa, SplitState& s)
+{
+    s.t = split3(-kTwoPi * b.y, kTwoPi * b.X);
+    s.q = split3(-kh * b.py, kh * b.px);
+    s.w = split3(b.wr, b.wi);
+    Z2 r;
+    split_force(hi2(s.w), kappa, s.f, r);
+    s.r = r.h;
+}
+
+// X, y, p, W0, 1/(1 + W0) and the force of b
+__device__ __forceinline__ void box_of_split(const SplitState& s, double ikh, double fk, Box<double>& b)
+{
+    b.X = kInvTwoPi * join_y(s.t);
+    b.y = -kInvTwoPi * join_x(s.t);
+    b.px = ikh * join_y(s.q);
+    b.py = -ikh * join_x(s.q);
+    b.wr = join_x(s.w);
+    b.wi = join_y(s.w);
+    const double ar = 1.0 + b.wr, inv = recip_nr(ar * ar + b.wi * b.wi);
+    b.rr = ar * inv;
+    b.ri = -b.wi * inv;
+    ray_force(b.wr, b.wi, b.rr, b.ri, fk, b.Fx, b.Fy);
+    wrap_cell<double, RT_RK4>(b);
+}
+
+// A trial step of the event location, any size h up to the scene's.
+static __device__ __noinline__ void rk4_split_step(const StepConst<double>& k, const Box<double>& s, double h,
+                                                   Box<double>& o)
+{
+    const double kh = kTwoPi * h, kappa = kh * kh * (k.fk * kInvTwoPi);
+    const float kappa_h = (float)kappa;
+    const F2 kp = {kappa_h, (float)(kappa - (double)kappa_h)};
+    SplitState a, b;
+    split_state(s, kh, kp, a);
+    split_step(a, kp, b);
+    o = s;
+    o.z = fma(h, s.pz, s.z);
+    box_of_split(b, 1.0 / kh, k.fk, o);
+}
+
 // One step of the scene's integrator of size h from s into o (for event
 // location: Phi_{theta h}(s) is one step of size theta h).
 template <class R, int INTEG>
 __device__ __forceinline__ void integ_step(const StepConst<R>& k, const Box<R>& s, R h, Box<R>& o, LaneStats& st)
 {
-    if constexpr (integ_of(INTEG) == RT_DP45) {
+    if constexpr (split_of(INTEG)) {
+        rk4_split_step(k, s, h, o);
+        st.evals += 4;
+        st.newton += 4;
+    } else if constexpr (integ_of(INTEG) == RT_DP45) {
         R e[4];
         dp45_step<R, INTEG>(k, s, h, o, e, st);
     } else if constexpr (integ_of(INTEG) == RT_RK4T) {
@@ -879,12 +951,13 @@ __device__ __forceinline__ void face_normal(int ev, R N[3])
 
 // Whether a trial step's end point needs a W0 solve: RK4 only continues W0
 // to its end point; the FP32 Dormand-Prince step has already solved it there
-// (or continued it exactly to FP32), as its last stage.  The FP64 path solves
+// (or continued it exactly to FP32), as its last stage, and the split double
+// precision step carries it there to more than FP64's rounding.  The FP64 path solves
 // again, as it always did, to keep its rays on the oracle's to 1e-12.
 template <class R, int INTEG>
 __host__ __device__ constexpr bool resolve_end()
 {
-    return !(sizeof(R) == 4 && integ_of(INTEG) == RT_DP45);
+    return !(sizeof(R) == 4 && integ_of(INTEG) == RT_DP45) && !split_of(INTEG);
 }
 
 // Root theta in (0, 1] of g_ev(Phi_{theta h}(b)) given its value g1 < 0 at
@@ -1479,6 +1552,7 @@ __device__ void air_segment(const DevScene& sc, Cold<R>& C, Box<R>& b, int& phas
             b.y = C.y;
             b.z = C.z;
             b.wr = b.wi = R(0);
+            if constexpr (sizeof(R) == 8 && !gauss_of(INTEG)) w0_seed(sc.cf, b.X, b.y, b.wr, b.wi);
             med_solve<R, INTEG>(k, b.X, b.y, b.wr, b.wi, b.rr, b.ri, b.Fx, b.Fy, st);
             // Snell's law in FP64 (a few operations per entry): sqrt(n^2 - |p_t|^2)
             // is ill-conditioned near grazing incidence; the index is scaled
@@ -1863,6 +1937,108 @@ __device__ __forceinline__ void box_step(const StepConst<R>& k, int64_t max_step
         box_step_into<R, INTEG>(k, max_steps, C, b, o, phase, surf, steps, st, safe);
         if (phase == PH_BOX) b = o;
     }
+}
+
+// ------------------------------------------------------------------------
+// The split double precision step (rt_split.cuh) in the integration loop.
+// ------------------------------------------------------------------------
+// A ray inside the cloak as the pool keeps it.  z moves linearly and is formed
+// where it is needed, from its value z0 at step `steps0` of the ray.
+struct SplitBox {
+    SplitState s;
+    double z0, dz;            // dz = h p_z
+    float cx, z0f, dzf;       // the cell (a whole number), and the same in FP32
+    int steps0;
+    double pad;
+};
+static_assert(sizeof(SplitBox) % 16 == 8, "consecutive entries on different banks");
+
+// The state a lane integrates and the pool keeps.
+template <class R, int INTEG> struct LoopBoxOf { using type = Box<R>; };
+template <> struct LoopBoxOf<double, RT_RK4 | kModeSplit> { using type = SplitBox; };
+template <class R, int INTEG> using LoopBox = typename LoopBoxOf<R, INTEG>::type;
+
+__device__ __forceinline__ void to_split(const DevScene& sc, const Box<double>& b, int steps, SplitBox& o)
+{
+    double wr = b.wr, wi = b.wi;
+    split_polish(sc.cd.kA, b.X, b.y, wr, wi);
+    Box<double> q = b;
+    q.wr = wr;
+    q.wi = wi;
+    split_state(q, sc.sp.kh, sc.sp.kappa, o.s);
+    o.cx = (float)b.cx;
+    o.z0 = b.z;
+    o.dz = sc.cd.h * b.pz;
+    o.z0f = (float)o.z0;
+    o.dzf = (float)o.dz;
+    o.steps0 = steps;
+}
+
+// n: steps taken since to_split
+__device__ __forceinline__ void from_split(const DevScene& sc, const SplitBox& o, int n, Box<double>& b)
+{
+    b.cx = (double)o.cx;
+    b.z = fma((double)n, o.dz, o.z0);
+    b.pz = o.dz * (kTwoPi * sc.sp.ikh);
+    b.cX = b.cy = b.cz = b.cpx = b.cpy = 0.0;
+    b.hc = sc.cd.h;
+    box_of_split(o.s, sc.sp.ikh, sc.cd.fk, b);
+}
+
+// One step in place of the pool entry e, whose state stays in shared memory
+// (held in registers through the step it spills: 82 local accesses a step
+// against some 30 shared ones).  A step that crosses a surface keeps its start
+// in e, as box_step does.  The grating's test is taken in FP32 on the leading
+// parts (their sum is exact where it is near zero).  The faces are tested only
+// where the ray may reach one (safe, see box_step_into), and in FP64 only
+// within kFaceNear of one: the conversions to FP64, which the lanes of a warp
+// reach at different steps, kept the FP64 pipe 36 % busy.
+constexpr float kFaceNear = 1e-4f;
+
+__device__ __forceinline__ void split_box_step(const DevScene& sc, F2 kappa, int64_t max_steps, Cold<double>& C,
+                                               SplitBox& e, int& phase, int& surf, int& steps, LaneStats& st,
+                                               int& safe)
+{
+    if (steps >= max_steps) {
+        phase = PH_GUARD;
+        return;
+    }
+    SplitState o;
+    split_step(e.s, kappa, o);
+    ++steps;
+    st.steps++;
+    const float g = (o.w.h.x - o.t.h.x) + (o.w.m.x - o.t.m.x);
+    if (safe > 0 && g >= 0.0f) {
+        --safe;
+    } else {
+        const StepConst<float>& kf = sc.cf;
+        const float i2pi = (float)kInvTwoPi;
+        const float x = fabsf(e.cx + i2pi * o.t.h.y), z = fabsf(fmaf((float)(steps - e.steps0), e.dzf, e.z0f));
+        const float d = fminf(kf.ytop + i2pi * o.t.h.x, kf.E2 - fmaxf(x, z));
+        if (g >= 0.0f && d > kFaceNear * (1.0f + kf.E2)) {
+            safe = (int)((d - 1e-5f * (1.0f + kf.E2)) * kf.isafe) - 1;
+        } else {
+            const StepConst<double>& k = sc.cd;
+            const double X = kInvTwoPi * join_y(o.t), y = -kInvTwoPi * join_x(o.t);
+            const double zd = fma((double)(steps - e.steps0), e.dz, e.z0);
+            const double gG = kInvTwoPi * (join_x(o.w) - join_x(o.t)), gT = k.ytop - y;
+            const double gXp = (k.E2 - (double)e.cx) - X, gXm = (k.E2 + (double)e.cx) + X, gZp = k.E2 - zd, gZm = k.E2 + zd;
+            if (!(gG >= 0.0 && gT >= 0.0 && gXp >= 0.0 && gXm >= 0.0 && gZp >= 0.0 && gZm >= 0.0)) {
+                C.g1[EV_GRATING] = gG;
+                C.g1[EV_TOP] = gT;
+                C.g1[EV_XP] = gXp;
+                C.g1[EV_XM] = gXm;
+                C.g1[EV_ZP] = gZp;
+                C.g1[EV_ZM] = gZm;
+                C.hs = k.h;
+                phase = PH_EVENT;
+                return;
+            }
+            safe = 0;
+        }
+    }
+    surf = EV_NONE;
+    e.s = o;
 }
 
 // ------------------------------------------------------------------------

@@ -52,15 +52,17 @@ template <class R, int INTEG>
 struct WaveShape {
     static constexpr bool kWide = sizeof(R) == 4 && integ_of(INTEG) == RT_DP45;
     static constexpr int kBlock = kWide ? 384 : 256;
-    static constexpr int kMinBlocks = (sizeof(R) == 4 && !kWide) ? 2 : 1;
-    static constexpr int P = kWide ? 576 : (sizeof(R) == 4 ? 384 : 320);
+    static constexpr int kMinBlocks = ((sizeof(R) == 4 && !kWide) || split_of(INTEG)) ? 2 : 1;
+    static constexpr int P = kWide ? 576 : (sizeof(R) == 4 ? 384 : (split_of(INTEG) ? 280 : 320));
 };
+
+static_assert((sizeof(Cold<double>) + sizeof(SplitBox) + 6) * 280 <= 115712, "two blocks of the split loop per SM");
 
 template <class R, int INTEG>
 constexpr size_t wave_smem_bytes()
 {
     constexpr int P = WaveShape<R, INTEG>::P;
-    return (sizeof(Cold<R>) + sizeof(Box<R>)) * P + 3 * sizeof(short) * P;
+    return (sizeof(Cold<R>) + sizeof(LoopBox<R, INTEG>)) * P + 3 * sizeof(short) * P;
 }
 
 // Bytes of the Fresnel branch queues of a launch of `grid` blocks.
@@ -190,14 +192,47 @@ __device__ __forceinline__ void wave_finish_sample(const Src& src, const DevScen
     src.pixel_done(C.scene);
 }
 
+// The integration task of the split double precision step: the rays' states
+// are SplitBoxes, stepped as in the general task of wave_loop.
+__device__ __forceinline__ void wave_split_task(const DevScene& sc, Cold<double>& C, int p, SplitBox* boxes, int m1,
+                                                int min_active, int& dest, LaneStats& st,
+                                                unsigned long long* iters)
+{
+    SplitBox& e = boxes[p >= 0 ? p : 0];
+    int phase = PH_IDLE, surf = EV_NONE, steps = 0;
+    if (p >= 0) {
+        phase = PH_BOX;
+        surf = C.surf;
+        steps = C.steps;
+    }
+    const int need = max(1, m1 - (32 - min_active));
+    const F2 kappa = sc.sp.kappa;
+    const int64_t max_steps = sc.max_steps;
+    int safe = 0;
+    for (int it = 0; it < kWaveTaskSteps; ++it) {
+#if RT_PROFILE
+        ++*iters;
+#endif
+        if (phase == PH_BOX) split_box_step(sc, kappa, max_steps, C, e, phase, surf, steps, st, safe);
+        if (__popc(__ballot_sync(0xffffffffu, phase == PH_BOX)) < need) break;
+    }
+    if (p >= 0) {
+        C.surf = surf;
+        C.steps = steps;
+        C.phase = phase;
+        dest = (phase == PH_BOX) ? WD_IN : WD_SRV;
+    }
+}
+
 template <class R, int INTEG, bool OPT, class Src>
 __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* counters, int min_active, WaveWait ww)
 {
     constexpr int P = WaveShape<R, INTEG>::P;
     extern __shared__ __align__(16) unsigned char wave_smem[];
     Cold<R>* cold = reinterpret_cast<Cold<R>*>(wave_smem);
-    Box<R>* boxes = reinterpret_cast<Box<R>*>(wave_smem + sizeof(Cold<R>) * P);
-    short* inq = reinterpret_cast<short*>(wave_smem + (sizeof(Cold<R>) + sizeof(Box<R>)) * P);
+    using LBox = LoopBox<R, INTEG>;
+    LBox* boxes = reinterpret_cast<LBox*>(wave_smem + sizeof(Cold<R>) * P);
+    short* inq = reinterpret_cast<short*>(wave_smem + (sizeof(Cold<R>) + sizeof(LBox)) * P);
     short* svq = inq + P;
     short* frq = svq + P;
     __shared__ WaveCtl Q;
@@ -300,8 +335,15 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
         Box<R> b;
         int phase = PH_IDLE, surf = EV_NONE, steps = 0;
         int dest = WD_NONE;
-        if (task == WT_INT) {
+        if (split_of(INTEG) && task == WT_INT) {
+            unsigned long long* iters = nullptr;
+#if RT_PROFILE
+            iters = &prof[2];
+#endif
+            if constexpr (split_of(INTEG)) wave_split_task(sc, C, p, boxes, m1, min_active, dest, st, iters);
+        } else if (task == WT_INT) {
             // ---- integrate ----
+            if constexpr (!split_of(INTEG)) {
             if (p >= 0) {
                 b = boxes[p];
                 phase = PH_BOX;
@@ -333,14 +375,19 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
                 C.phase = phase;
                 dest = (phase == PH_BOX) ? WD_IN : WD_SRV;
             }
+            }
         } else {
             // ---- serve ----
             if (p >= 0) {
                 if (!fresh) {
-                    b = boxes[p];
                     phase = C.phase;
                     surf = C.surf;
                     steps = C.steps;
+                    // (a step that crossed a surface is counted, but its start is kept)
+                    if constexpr (split_of(INTEG))
+                        from_split(sc, boxes[p], steps - boxes[p].steps0 - (phase == PH_EVENT ? 1 : 0), b);
+                    else
+                        b = boxes[p];
                 }
                 while (phase != PH_BOX && phase != PH_EXIT) {
                     if (phase == PH_EVENT || phase == PH_GUARD)
@@ -376,7 +423,8 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
                     }
                 }
                 if (phase == PH_BOX) {
-                    boxes[p] = b;
+                    if constexpr (split_of(INTEG)) to_split(src.scene(C.scene), b, steps, boxes[p]);
+                    else boxes[p] = b;
                     C.surf = surf;
                     C.steps = steps;
                     C.phase = PH_BOX;
@@ -401,6 +449,11 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
     }
     __syncthreads();
 
+    // the split step evaluates four times and solves or continues W0 four times
+    if constexpr (split_of(INTEG)) {
+        st.evals += 4 * st.steps;
+        st.newton += 4 * st.steps;
+    }
     // counters: per-thread integration counters and the pool's per-pixel ones
     uint32_t v[11] = {0u, st.steps, st.evals, st.newton, 0u, st.refine, 0u, 0u, 0u, 0u, 0u};
     for (int p = threadIdx.x; p < P; p += blockDim.x) {

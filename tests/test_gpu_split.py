@@ -1,0 +1,73 @@
+"""The FP64 RK4 step in two- and three-float arithmetic (rt_split.cuh) against
+the general FP64 step, which the per-lane loop takes, and against the oracle's
+paths, at the edges of the step's bounds and just past them."""
+import numpy as np
+import pytest
+
+from paper_1012_5107_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def render(rt, torch, p, variant):
+    sc = rt.Scene(p)
+    sc.set_launch(variant, 0)
+    n = sc.height * sc.wout * sc.spp
+    rgb = torch.zeros(sc.shape, dtype=torch.float32, device="cuda")
+    rec = torch.zeros(n * 80, dtype=torch.uint8, device="cuda")
+    sc.render(rgb, rec=rec)
+    torch.cuda.synchronize()
+    return rgb.cpu().numpy(), rt.records_to_numpy(rec), sc.stats()
+
+
+# Both steps round at about 1e-16 a step; over some 1000 steps and the
+# amplification of the rays that graze the grating, exits agree to 1e-12 on
+# nearly all rays, and the bar is the one of the launch variants (1e-10).
+@pytest.mark.parametrize("over", [
+    dict(),
+    dict(A=0.0),                                        # W0 = 0 everywhere
+    dict(A=1e-6),                                       # a force far below the rounding of the momentum
+    dict(A=0.0477),                                     # kA = 0.2997, the largest the step takes
+    dict(A=0.048, width=24, height=20),                 # just past it: the general step
+    dict(h=1.0 / 110.0, A=0.02),                        # |D| = 0.0653 at n_max: the general step
+    dict(h=1.0 / 117.0, A=0.02),                        # 0.0614: within the bound
+    dict(h=1.0 / 900.0, width=16, height=12),           # short steps
+    dict(H=7.9, E=24.0, cam_dist=30.0, width=24, height=20),   # |W0| = 1e-22 at the box's top
+    dict(H=8.1, E=24.0, cam_dist=30.0, width=12, height=8),    # past the bound on the box's height
+    dict(H=0.11, E=6.0),                                # a box barely above the crests
+    dict(E=0.7, elev_deg=12.0),                         # faces within a few steps of one another
+    dict(E=32.0, cam_dist=40.0, width=24, height=20),
+    dict(max_steps=50),                                 # the guard inside the cloak
+    dict(max_bounces=0),
+    dict(azim_deg=90.0, elev_deg=15.0),                 # along the grooves
+    dict(width=7, height=5, spp=3, Lambda=0.6, A=0.02, E=4.8, H=1.2, h=0.003, cam_dist=7.2, bg_cell=0.3),
+])
+def test_split_step_equals_general_step(over):
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    p = inputs.base_scene(**{**dict(width=40, height=32, spp=1, precision=1), **over})
+    a_rgb, a, a_st = render(rt, torch, p, 0)
+    b_rgb, b, b_st = render(rt, torch, p, 3)
+    assert a_st["rays"] == b_st["rays"] and a_st["steps"] == b_st["steps"] and a_st["status"] == b_st["status"]
+    assert b_st["evals"] >= 4 * b_st["steps"]
+    for name in ("status", "bounces", "events", "steps"):
+        assert np.array_equal(a[name], b[name]), name
+    assert np.abs(a["pos"] - b["pos"]).max() <= 1e-10 * p["Lambda"]
+    assert np.abs(a["dir"] - b["dir"]).max() <= 1e-10
+    assert np.array_equal(a_rgb, b_rgb)
+
+
+def test_split_render_repeats_and_matches_for_every_grouping():
+    """The grouping of rays into warps changes no bit of the records."""
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    p = inputs.base_scene(width=72, height=50, spp=4, seed=5, precision=1)
+    sc = rt.Scene(p)
+    out = []
+    for min_active in (1, 16, 28, 32, 28):
+        sc.set_launch(3, min_active)
+        rec = torch.zeros(72 * 50 * 4 * 80, dtype=torch.uint8, device="cuda")
+        rgb = torch.zeros(sc.shape, dtype=torch.float32, device="cuda")
+        sc.render(rgb, rec=rec)
+        out.append(rec.cpu().numpy())
+    assert all(np.array_equal(out[0], o) for o in out[1:])
