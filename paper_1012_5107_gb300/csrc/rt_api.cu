@@ -6,6 +6,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <atomic>
+#include <mutex>
 
 #include "rt_internal.h"
 
@@ -19,6 +21,48 @@ void set_error(const char* fmt, ...)
     va_start(ap, fmt);
     vsnprintf(g_err, sizeof g_err, fmt, ap);
     va_end(ap);
+}
+
+// One pool per device, made at its first use.
+constexpr int kScratchDevices = 64;
+static std::mutex g_scratch_mutex;
+static cudaMemPool_t g_scratch_pool[kScratchDevices];
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t stream)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= kScratchDevices) return cudaMallocAsync(p, bytes, stream);
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lock(g_scratch_mutex);
+        if (!g_scratch_pool[dev]) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t made;
+            e = cudaMemPoolCreate(&made, &props);
+            if (e != cudaSuccess) return e;
+            uint64_t keep = kScratchKeep;
+            e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) {
+                cudaMemPoolDestroy(made);
+                return e;
+            }
+            g_scratch_pool[dev] = made;
+        }
+        pool = g_scratch_pool[dev];
+    }
+    return cudaMallocFromPoolAsync(p, bytes, pool, stream);
+}
+
+void scratch_trim()
+{
+    std::lock_guard<std::mutex> lock(g_scratch_mutex);
+    for (cudaMemPool_t pool : g_scratch_pool)
+        if (pool) cudaMemPoolTrimTo(pool, 0);
 }
 
 }  // namespace grt
@@ -62,7 +106,10 @@ struct rt_scene {
     cudaEvent_t done;
     bool rendered;
     WaitLimit wait;           // bounds of the wavefront loop's waits (rt_scene_set_wait_limit)
+    bool counted;             // in g_scenes
 };
+
+static std::atomic<int> g_scenes{0};
 
 static int current_device(int* dev)
 {
@@ -354,6 +401,8 @@ int rt_create_scene(const rt_scene_desc* desc, rt_scene** out)
     }
     s->dev.tex = s->d_tex;
     s->grid = (bps > 0 ? bps : 1) * nsm;
+    g_scenes.fetch_add(1);
+    s->counted = true;
     *out = s;
     return RT_OK;
 }
@@ -370,6 +419,8 @@ void rt_destroy_scene(rt_scene* s)
     if (s->d_pcnt) cudaFree(s->d_pcnt);
     if (s->d_branch) cudaFree(s->d_branch);
     if (s->done) cudaEventDestroy(s->done);
+    // the last scene gives the correlation calls' scratch back
+    if (s->counted && g_scenes.fetch_sub(1) == 1) scratch_trim();
     free(s);
 }
 
@@ -591,9 +642,9 @@ int rt_xcorr(const float* d_f, const float* d_g, int32_t height, int32_t width, 
     Windows win;
     fov_windows(width, hfov_deg, fov_deg, n_fov, &win);
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t bytes = xcorr_scratch_bytes(height, width, channels);
+    const size_t bytes = xcorr_scratch_bytes(height, width, channels, n_fov);
     void* partial = nullptr;
-    if (bytes) RT_CK(cudaMallocAsync(&partial, bytes, st));
+    if (bytes) RT_CK(scratch_alloc(&partial, bytes, st));
     cudaError_t e = launch_xcorr(d_f, d_g, height, width, channels, win, partial, d_out, st);
     cudaError_t e2 = bytes ? cudaFreeAsync(partial, st) : cudaSuccess;
     RT_CK(e);

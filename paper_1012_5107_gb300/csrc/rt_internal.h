@@ -110,13 +110,18 @@ cudaError_t launch_render(const DevScene& sc, int precision, int variant, int mi
 cudaError_t launch_medium(int precision, double kA, double Lambda, const double* xy, int64_t n, double* out,
                           cudaStream_t stream);
 
-// Cross-correlation: column moments per row chunk (nchunks x W*C double4,
-// padded to 256 bytes), then window slices (kXcorrTailBytes), then C.
-// `scratch` holds xcorr_scratch_bytes(H, W, C) bytes, 256-byte aligned (none
-// for the small images that one block takes).
-constexpr size_t kXcorrTailBytes = 129 * 1024;
-int xcorr_chunks(int H);
-size_t xcorr_scratch_bytes(int H, int W, int C);
+// Cross-correlation: moments per window and block, then C.  `scratch` holds
+// xcorr_scratch_bytes(...) bytes, at most kXcorrScratch (none for the small
+// images that one block takes).
+constexpr size_t kXcorrScratch = (size_t)5 << 18;
+size_t xcorr_scratch_bytes(int H, int W, int C, int n_fov);
+// Scratch of the correlation calls, in stream order, from a pool of the
+// library's own that keeps up to kScratchKeep bytes between calls (the default
+// pool gives everything back at each synchronisation: 0.2 ms for the next
+// call).  scratch_trim gives the kept memory back.
+constexpr size_t kScratchKeep = (size_t)64 << 20;
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t stream);
+void scratch_trim();
 cudaError_t launch_xcorr(const float* f, const float* g, int H, int W, int C, const Windows& win, void* scratch,
                          double* out, cudaStream_t stream);
 

@@ -337,8 +337,8 @@ extern "C" int rt_xcorr_map(const float* const* d_f, const float* const* d_g, in
                                ~(size_t)255;
     const size_t ncol = (size_t)npc * ncc * nshift;
     const size_t part_bytes = chunk_bytes + sizeof(double) * ncol;
-    cudaError_t e = cudaMallocAsync((void**)&stats, sizeof(double) * 3 * npc, st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&partial, part_bytes, st);
+    cudaError_t e = scratch_alloc((void**)&stats, sizeof(double) * 3 * npc, st);
+    if (e == cudaSuccess) e = scratch_alloc((void**)&partial, part_bytes, st);
     if (e == cudaSuccess) {
         xmap_moment_rows<<<dim3(mchunks, n_pairs), kMomBlock, 0, st>>>(im, height, width, channels, j0, j1, mchunks,
                                                                         partial);

@@ -5,11 +5,10 @@
 // own pool and forbid allocations behind its back, and latency-bound loops
 // in which an allocation call (which can synchronise the device or take a
 // driver lock) is not acceptable.  This entry point runs the same
-// kernels as rt_xcorr but keeps their scratch -- the per-chunk column
-// moments and the window slices -- in the file-scope device array below
-// instead of allocating it.
+// kernels as rt_xcorr but keeps their scratch -- the moments per window and
+// block -- in the file-scope device array below instead of allocating it.
 //
-// The array is a fixed 16 MiB (and the slices' 129 KiB) that every GPU
+// The array is a fixed 1.25 MiB that every GPU
 // which loads the library holds until the process exits.  Host code must not pass the array's name to a
 // kernel: in host code it names a host-side stand-in, not device memory.  The
 // device address is taken with cudaGetSymbolAddress, once per device, with
@@ -17,6 +16,7 @@
 // and kept for the life of the process: a cudaDeviceReset of that device
 // invalidates it (the module is loaded again, possibly elsewhere), so the
 // entry point must not be used on a device after resetting it.
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 
@@ -24,16 +24,10 @@
 
 namespace grt {
 
-struct alignas(32) NoallocMoments {
-    double v[4];
-};
-
-// Largest column-moment scratch in 32-byte moment records: 16 MiB; the array
-// adds the window slices and the padding between the two.
+// Largest image taken: min(ceil(height / 64), 64) * width * channels.
 constexpr size_t kNoallocMoments = (size_t)16 << 20 >> 5;
-constexpr size_t kNoallocRecords = kNoallocMoments + (kXcorrTailBytes + 256) / sizeof(NoallocMoments);
 
-static __device__ __align__(256) NoallocMoments g_xcorr_scratch[kNoallocRecords];
+static __device__ __align__(256) unsigned char g_xcorr_scratch[kXcorrScratch];
 
 constexpr int kNoallocMaxDevices = 64;
 static std::mutex g_noalloc_mutex;
@@ -72,12 +66,11 @@ extern "C" int rt_xcorr_noalloc(const float* d_f, const float* d_g, int32_t heig
     if (!(hfov_deg > 0.0 && hfov_deg < 180.0)) { set_error("hfov_deg must be in (0, 180)"); return RT_EINVAL; }
     for (int q = 0; q < n_fov; ++q)
         if (!(fov_deg[q] >= 0.0)) { set_error("fov_deg must be >= 0"); return RT_EINVAL; }
-    const size_t need = (size_t)xcorr_chunks(height) * (size_t)width * (size_t)channels;
-    if (need > kNoallocMoments || xcorr_scratch_bytes(height, width, channels) > sizeof(g_xcorr_scratch)) {
-        set_error("rt_xcorr_noalloc: %d x %d x %d images need %zu bytes of scratch; the fixed scratch holds %zu "
-                  "bytes (min(ceil(height / 64), 64) * width * channels must be <= %zu)",
-                  height, width, channels, need * sizeof(NoallocMoments), kNoallocMoments * sizeof(NoallocMoments),
-                  kNoallocMoments);
+    const size_t need = (size_t)std::min((height + 63) / 64, 64) * (size_t)width * (size_t)channels;
+    if (need > kNoallocMoments || xcorr_scratch_bytes(height, width, channels, n_fov) > sizeof(g_xcorr_scratch)) {
+        set_error("rt_xcorr_noalloc: %d x %d x %d images are too large for the fixed scratch "
+                  "(min(ceil(height / 64), 64) * width * channels must be <= %zu)",
+                  height, width, channels, kNoallocMoments);
         return RT_EINVAL;
     }
     int dev = 0;

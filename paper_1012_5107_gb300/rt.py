@@ -145,8 +145,9 @@ def _check(rc: int):
 
 def _stream(stream) -> int | None:
     if stream is None:
+        # the raw handle: torch.cuda.current_stream() builds a Stream object
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

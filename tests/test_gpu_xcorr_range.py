@@ -1,0 +1,63 @@
+"""rt_xcorr over the ranges its three-float sums take and past them (where a
+block sums in FP64), and its column tiles, against Eqs. 14-15 in FP64."""
+import math
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def columns(W, hfov, fov):
+    px = 2.0 * (np.arange(W) + 0.5) / W - 1.0
+    a = np.degrees(np.arctan(np.abs(px) * math.tan(math.radians(0.5 * hfov))))
+    return np.nonzero(a <= 0.5 * fov + 1e-9)[0]
+
+
+def c00(f, g, cols):
+    f, g = f[:, cols].astype(np.float64), g[:, cols].astype(np.float64)
+    f, g = f - f.mean((0, 1)), g - g.mean((0, 1))
+    num, den = (f * g).sum((0, 1)), (f * f).sum((0, 1))
+    return np.append(num / den, num.sum() / den.sum())
+
+
+# FP64 moments of N values lose about N^(1/2) 1e-16 times the ratio of the
+# mean square to the variance (at most 1e2 here): 1e-11 covers the largest.
+@pytest.mark.parametrize("H,W,C,scale", [
+    (512, 512, 3, 1.0), (7, 9721, 3, 1.0), (1, 9999, 4, 1.0), (2000, 22, 3, 1.0), (1030, 65, 1, 1.0),
+    (33, 9729, 1, 1.0),                                  # one column past kXcorrBlocks tiles of 32
+    (96, 70, 2, 2.0 ** -39), (96, 70, 2, 2.0 ** 59),     # the edges of the three-float range
+    (96, 70, 2, 1e-30), (96, 70, 2, 1e25),               # products past FP32's range: FP64
+])
+def test_xcorr_ranges(H, W, C, scale):
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    rng = np.random.default_rng([H, W, C])
+    f = (np.round(4.0 * rng.random((H, W, C))) * 0.25 + 0.1 * rng.random((H, W, C))).astype(np.float32)
+    g = (0.7 * f + 0.3 * rng.random((H, W, C))).astype(np.float32)
+    f[0, 0, 0] = 0.0
+    f, g = (f * np.float32(scale)).astype(np.float32), (g * np.float32(scale)).astype(np.float32)
+    fovs = [0.0, 10.0, 25.0, 50.0]
+    tf, tg = torch.from_numpy(f).cuda(), torch.from_numpy(g).cuda()
+    out = rt.xcorr(tf, tg, fovs, 50.0).cpu().numpy()
+    again = rt.xcorr(tf, tg, fovs, 50.0).cpu().numpy()
+    assert np.array_equal(out, again, equal_nan=True)
+    for q, fov in enumerate(fovs):
+        cols = columns(W, 50.0, fov)
+        if H * len(cols) > 1:                            # one pixel has no variance: 0/0
+            assert np.abs(out[q] - c00(f, g, cols)).max() < 1e-11
+        else:
+            assert np.isnan(out[q]).all()
+
+
+def test_xcorr_infinities_and_nan():
+    """A value that is not finite spoils its own windows and channel only, as FP64 sums do."""
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    rng = np.random.default_rng(3)
+    f, g = (rng.random((64, 96, 3)).astype(np.float32) for _ in range(2))
+    g[5, 0, 1] = np.inf                                 # outside the inner window
+    f[9, 95, 2] = np.nan
+    out = rt.xcorr(torch.from_numpy(f).cuda(), torch.from_numpy(g).cuda(), [10.0, 50.0], 50.0).cpu().numpy()
+    assert np.isfinite(out[0]).all()
+    assert np.isfinite(out[1, 0]) and not np.isfinite(out[1, 1]) and np.isnan(out[1, 2]) and not np.isfinite(out[1, 3])
