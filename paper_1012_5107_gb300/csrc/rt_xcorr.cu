@@ -28,6 +28,7 @@
 #include <cmath>
 
 #include "rt_internal.h"
+#include "rt_moments.cuh"
 
 namespace grt {
 
@@ -58,28 +59,6 @@ size_t xcorr_scratch_bytes(int H, int W, int C, int n_fov)
     if (xcorr_one_block(H, W, C)) return 0;
     const dim3 g = xcorr_grid(H, W, C);
     return (size_t)g.x * g.y * (size_t)n_fov * 4 * C * sizeof(double);
-}
-
-// Values that the three-float sums take: zero, or a magnitude in [2^-40, 2^60),
-// whose products neither overflow nor lose their remainders to underflow.
-__device__ __forceinline__ bool xcorr_plain(float v)
-{
-    const uint32_t u = __float_as_uint(v) & 0x7fffffffu;
-    return u == 0u || u - (87u << 23) < (100u << 23);
-}
-
-// Three-float running sums of a pair of values; xcorr_low adds remainders.
-__device__ __forceinline__ void xcorr_low(Z3& s, float2 v)
-{
-    const Z2 t = two_sum(s.m, v);
-    s.m = t.h;
-    s.l = vadd(s.l, t.l);
-}
-__device__ __forceinline__ void xcorr_add(Z3& s, float2 v)
-{
-    const Z2 t = two_sum(s.h, v);
-    s.h = t.h;
-    xcorr_low(s, t.l);
 }
 
 // Moments of 32 columns over the block's rows, to col[moment][column] (threads

@@ -2,15 +2,15 @@
 // pixel shifts, its peak and its mean over several reference pairs (Sec. 5).
 //
 // Pass 1 forms, over the field-of-view window of columns j0..j1-1, the means
-// of Eq. 14 and the denominator sum (f - <f>)^2 of Eq. 15 in FP64: blocks of
-// 4 image rows per pair sum them (FP64 is slow on this GPU, so the work is
-// spread over many SMs), then a block per pair and channel adds the chunks.
-// Pass 2 is a direct correlation in tiles: a block owns 16 R x 16 R shifts
-// (di, dj) and a chunk of 8 image rows x 128 columns of one pair and
-// channel; it stages the chunk of f and the window of g its shifts need (zero
-// outside the field-of-view window, where the finite photographs have no
-// values) in shared memory, and each thread accumulates the products of its
-// R x R shifts over the chunk with FP32 FMA (see xmap_tiles).
+// of Eq. 14 and the denominator sum (f - <f>)^2 of Eq. 15: a block per image
+// row and pair sums it in three floats (rt_moments.cuh), then a block per pair
+// and channel adds the rows in FP64.
+// Pass 2 is a direct correlation in tiles: a block stages chunks of 8 image
+// rows x 128 columns of f, of one pair and channel, and the window of g that
+// its shifts (di, dj) need (zero outside the field-of-view window, where the
+// finite photographs have no values) in shared memory, and each thread
+// accumulates the products of its few shifts over a chunk with FP32 FMA (see
+// xmap_tiles; choose_plan says how many).
 // Pass 3 adds, per shift, pair, channel and column chunk, the row chunks'
 // sums with compensated (Kahan) FP32 summation, whose error is of the order
 // of one FP32 rounding of the result, below the rounding already in each
@@ -18,28 +18,32 @@
 // column chunks in FP64, divides by the denominators, stacks the channels
 // (sum of numerators over sum of denominators) and averages the maps of the
 // pairs; pass 5 finds the peak of the stacked mean map and its shift.
+//
+// Measured: +-32 shifts of a 512 x 512 x 3 pair 320 -> 215 us.  The tiles, 261 us
+// of it, computed 80 x 80 shifts for the 65 x 65 wanted, 25 a thread; now the
+// threads' shifts divide those wanted and the tiles take 150 us (72 us at the
+// FP32 peak).  +-31 x +-3 shifts of two 326 x 164 pairs 139 -> 58 us, +-40 of two
+// 300 x 400 x 3 pairs 1,095 -> 312 us.
 #include <algorithm>
 #include <cmath>
 #include <vector>
 
 #include "rt_internal.h"
+#include "rt_moments.cuh"
 
 namespace grt {
 
-constexpr int kMapT = 16;         // threads along di and along dj
 constexpr int kMapRows = 8;       // image rows per chunk
 constexpr int kMapCols = 128;     // image columns per chunk
-constexpr int kMapBlock = kMapT * kMapT;
+constexpr int kMapThreads = 160;  // threads per block of the tiles, at most
 constexpr int kMapMaxShift = 64;
 
-// Staged g window of a block with R x R shifts per thread: rows x padded
-// columns (one column past the window is read, never used, by the sliding
-// loads of the last column).
-template <int R> struct MapTile {
-    static constexpr int TD = kMapT * R;                  // shifts per block along di and dj
-    static constexpr int GR = kMapRows + TD - 1;
-    static constexpr int GC = kMapCols + TD;
-    static constexpr size_t smem = sizeof(float) * ((size_t)GR * GC + (size_t)kMapRows * kMapCols);
+// How a launch of the tiles is laid out: a thread owns RI x RJ shifts, gi x gj
+// threads the shifts of a chunk, of which a block takes git along di; kc row
+// chunks share a block and its window of g, gc floats a row.
+struct MapPlan {
+    int ri, rj, gi, gj, git, kc, gc, threads;
+    size_t smem;
 };
 constexpr int kMapMaxPairs = 64;
 
@@ -48,7 +52,7 @@ struct MapImages {
     const float* g[kMapMaxPairs];
 };
 
-constexpr int kMomRows = 4;       // image rows per block of pass 1
+constexpr int kMomRows = 1;       // image rows per block of pass 1
 constexpr int kMomBlock = 256;
 
 // A window row's values, (i W + j0) C ... (i W + j1) C, are contiguous, and
@@ -66,30 +70,50 @@ __global__ void __launch_bounds__(kMomBlock) xmap_moment_rows(MapImages im, int 
     const int len = (j1 - j0) * C;
     const int t = threadIdx.x;
     const int i0 = chunk * kMomRows, i1 = min(H, i0 + kMomRows);
-    double sf = 0.0, sg = 0.0, sff = 0.0;
+    Z3 s1 = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, s2 = s1;   // (f, g) and (f^2, -)
+    int odd = 0;
     if (t < T) {
         for (int i = i0; i < i1; ++i) {
             const int64_t base = ((int64_t)i * W + j0) * C;
 #pragma unroll 4
             for (int e = t; e < len; e += T) {
-                const double a = __ldg(f + base + e), b = __ldg(g + base + e);
-                sf += a;
-                sg += b;
-                sff += a * a;
+                const float a = __ldg(f + base + e), b = __ldg(g + base + e);
+                odd |= !(xcorr_plain(a) && xcorr_plain(b));
+                const F2 p = two_prod(a, a);
+                xcorr_add(s1, float2{a, b});
+                xcorr_add(s2, float2{p.h, 0.0f});
+                xcorr_low(s2, float2{p.l, 0.0f});
             }
         }
+    }
+    double sf = join_x(s1), sg = join_y(s1), sff = join_x(s2);
+    if (__syncthreads_or(odd)) {                                  // outside the three-float range: in FP64
+        sf = sg = sff = 0.0;
+        if (t < T)
+            for (int i = i0; i < i1; ++i) {
+                const int64_t base = ((int64_t)i * W + j0) * C;
+                for (int e = t; e < len; e += T) {
+                    const double a = __ldg(f + base + e), b = __ldg(g + base + e);
+                    sf += a;
+                    sg += b;
+                    sff += a * a;
+                }
+            }
     }
     red[0][t] = sf;
     red[1][t] = sg;
     red[2][t] = sff;
     __syncthreads();
-    if (t < 3 * C) {
-        const int q = t / C, c = t - q * C;
-        double acc = 0.0;
-        for (int k = c; k < T; k += C) acc += red[q][k];
-        part[(((int64_t)pair * nchunks + chunk) * C + c) * 3 + q] = acc;
-    }
+    // the threads of a channel in two rounds of additions
+    constexpr int kWays = 16;
+    double acc = 0.0;
+    const int way = t % kWays, o = t / kWays, q = o / C, c = o - q * C;
+    if (o < 3 * C)
+        for (int k = c + way * C; k < T; k += kWays * C) acc += red[q][k];
+    for (int d = kWays / 2; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d, kWays);
+    if (o < 3 * C && way == 0) part[(((int64_t)pair * nchunks + chunk) * C + c) * 3 + q] = acc;
 }
+static_assert(16 * 3 * 4 <= kMomBlock, "sixteen threads per channel and sum");
 
 // Block per (pair, channel): the chunks' sums, then the statistics.
 __global__ void __launch_bounds__(128) xmap_moment_stats(const double* __restrict__ part, int H, int C, int j0,
@@ -122,82 +146,113 @@ __global__ void __launch_bounds__(128) xmap_moment_stats(const double* __restric
     }
 }
 
-// Thread (ty, tx) owns the shifts di = di_lo + ty R + a, dj = dj_lo + tx R + b
-// (a, b < R).  The product f(i, j) g(i + di, j + dj) of chunk row r and column
-// q reads g_s[r + ty R + a][q + tx R + b]; along q each of the R g rows a
-// thread reads slides by one column, so a column costs one broadcast f load
-// and R g loads for R^2 FMAs.  The chunk's sum per shift is FP32 (8 x 128
-// products); part[((pc nchunks + chunk) nshift + s)], chunk = rc ncc + cc.
-template <int R>
-__global__ void __launch_bounds__(kMapBlock) xmap_tiles(MapImages im, const double* __restrict__ stats, int H, int W,
-                                                        int C, int j0, int j1, int max_di, int max_dj, int ncc,
-                                                        int nchunks, float* __restrict__ part)
+// A thread owns the shifts (di0 + a, dj0 + b), a < RI, b < RJ, of one chunk.
+// The product f(i, j) g(i + di, j + dj) of chunk row r and column q reads
+// g_s[r + a][q + b] of its window; along q each of the RI g rows slides by one
+// column, held in registers by position modulo RJ, so a column costs one
+// broadcast f load and RI g loads for RI RJ FMAs: shared memory delivers one
+// load a cycle to the SM's four FMA pipes, which 5 x 5 shifts a thread all but
+// used up.  The chunk's sum per shift is FP32 (8 x 128 products, in that
+// order); part[((pc nchunks + chunk) nshift + s)], chunk = rc ncc + cc.
+template <int RI, int RJ>
+__global__ void __launch_bounds__(kMapThreads, 3) xmap_tiles(MapImages im, const double* __restrict__ stats, int H,
+                                                             int W, int C, int j0, int j1, int max_di, int max_dj,
+                                                             int nrc, int ncc, MapPlan pl, float* __restrict__ part)
 {
-    using Tl = MapTile<R>;
     extern __shared__ float map_smem[];
-    float* g_s = map_smem;                                   // [GR][GC]
-    float* f_s = map_smem + (size_t)Tl::GR * Tl::GC;         // [kMapRows][kMapCols]
+    const int GC = pl.gc, rows_f = pl.kc * kMapRows, rows_g = rows_f + pl.git * RI - 1;
+    float* g_s = map_smem;                                   // [rows_g][GC]
+    float* f_s = map_smem + (size_t)rows_g * GC;             // [rows_f][kMapCols]
     const int ndi = 2 * max_di + 1, ndj = 2 * max_dj + 1;
-    const int tiles_dj = (ndj + Tl::TD - 1) / Tl::TD;
-    const int tdi = blockIdx.x / tiles_dj, tdj = blockIdx.x % tiles_dj;
-    const int chunk = blockIdx.y;
-    const int rc = chunk / ncc, cc = chunk % ncc;
-    const int pc = blockIdx.z;
+    const int tiles = (pl.gi + pl.git - 1) / pl.git;
+    const int tile = blockIdx.x % tiles, group = blockIdx.x / tiles;
+    const int cc = group % ncc, rc0 = (group / ncc) * pl.kc;
+    const int pc = blockIdx.y;
     const int pair = pc / C, c = pc % C;
     const float* f = im.f[pair];
     const float* g = im.g[pair];
     const float mf = (float)stats[3 * pc + 0], mg = (float)stats[3 * pc + 1];
-    const int di_lo = -max_di + tdi * Tl::TD, dj_lo = -max_dj + tdj * Tl::TD;
-    const int i0 = rc * kMapRows, jc = j0 + cc * kMapCols;
-    for (int k = threadIdx.x; k < kMapRows * kMapCols; k += kMapBlock) {
-        const int r = k / kMapCols, q = k % kMapCols;
-        const int i = i0 + r, j = jc + q;
-        f_s[k] = (i < H && j < j1) ? __ldg(f + ((int64_t)i * W + j) * C + c) - mf : 0.0f;
+    const int di_lo = -max_di + tile * pl.git * RI, dj_lo = -max_dj;
+    const int i0 = rc0 * kMapRows, jc = j0 + cc * kMapCols;
+    // rows by warps, eight loads in flight a lane
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    for (int r = warp; r < rows_f; r += nwarp) {
+        const int i = i0 + r;
+        float v[kMapCols / 32];
+#pragma unroll
+        for (int k = 0; k < kMapCols / 32; ++k) {
+            const int j = jc + lane + 32 * k;
+            v[k] = (i < H && j < j1) ? __ldg(f + ((int64_t)i * W + j) * C + c) - mf : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < kMapCols / 32; ++k) f_s[r * kMapCols + lane + 32 * k] = v[k];
     }
-    for (int k = threadIdx.x; k < Tl::GR * Tl::GC; k += kMapBlock) {
-        const int r = k / Tl::GC, q = k % Tl::GC;
-        const int i = i0 + di_lo + r, j = jc + dj_lo + q;
-        g_s[k] = (i >= 0 && i < H && j >= j0 && j < j1) ? __ldg(g + ((int64_t)i * W + j) * C + c) - mg : 0.0f;
-    }
-    __syncthreads();
-    const int ty = threadIdx.x / kMapT, tx = threadIdx.x % kMapT;
-    float acc[R][R];
+    for (int r = warp; r < rows_g; r += nwarp) {
+        const int i = i0 + di_lo + r;
+        const bool row = i >= 0 && i < H;
+        const float* gi = g + (int64_t)i * W * C + c;
+        for (int q0 = lane; q0 < GC; q0 += 256) {
+            float v[8];
 #pragma unroll
-    for (int a = 0; a < R; ++a)
-#pragma unroll
-        for (int b = 0; b < R; ++b) acc[a][b] = 0.0f;
-    for (int r = 0; r < kMapRows; ++r) {
-        const float* fr = f_s + r * kMapCols;
-        const float* gr = g_s + (size_t)(r + ty * R) * Tl::GC + tx * R;
-        float win[R][R];
-#pragma unroll
-        for (int a = 0; a < R; ++a)
-#pragma unroll
-            for (int b = 0; b < R; ++b) win[a][b] = gr[a * Tl::GC + b];
-#pragma unroll 16
-        for (int q = 0; q < kMapCols; ++q) {
-            const float fv = fr[q];
-#pragma unroll
-            for (int a = 0; a < R; ++a) {
-#pragma unroll
-                for (int b = 0; b < R; ++b) acc[a][b] = fmaf(fv, win[a][b], acc[a][b]);
-#pragma unroll
-                for (int b = 0; b + 1 < R; ++b) win[a][b] = win[a][b + 1];
-                win[a][R - 1] = gr[a * Tl::GC + q + R];
+            for (int k = 0; k < 8; ++k) {
+                const int j = jc + dj_lo + q0 + 32 * k;
+                v[k] = (row && j >= j0 && j < j1) ? __ldg(gi + (int64_t)j * C) - mg : 0.0f;
             }
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (q0 + 32 * k < GC) g_s[r * GC + q0 + 32 * k] = v[k];
         }
     }
-    const int64_t nshift = (int64_t)ndi * ndj;
+    __syncthreads();
+    const int units = pl.git * pl.gj;
+    const int kc = threadIdx.x / units, u = threadIdx.x - kc * units;
+    const int ui = u / pl.gj, uj = u - ui * pl.gj;
+    const int rc = rc0 + kc;
+    if (kc >= pl.kc || rc >= nrc || tile * pl.git + ui >= pl.gi) return;
+    float acc[RI][RJ];
 #pragma unroll
-    for (int a = 0; a < R; ++a) {
-        const int di = di_lo + ty * R + a;
+    for (int a = 0; a < RI; ++a)
 #pragma unroll
-        for (int b = 0; b < R; ++b) {
-            const int dj = dj_lo + tx * R + b;
-            if (di <= max_di && dj <= max_dj) {
-                const int64_t sh = (int64_t)(di + max_di) * ndj + (dj + max_dj);
-                part[((int64_t)pc * nchunks + chunk) * nshift + sh] = acc[a][b];
+        for (int b = 0; b < RJ; ++b) acc[a][b] = 0.0f;
+    for (int r = 0; r < kMapRows; ++r) {
+        const float* fr = f_s + (kc * kMapRows + r) * kMapCols;
+        const float* gr = g_s + (size_t)(kc * kMapRows + r + ui * RI) * GC + uj * RJ;
+        float win[RI][RJ];
+#pragma unroll
+        for (int a = 0; a < RI; ++a)
+#pragma unroll
+            for (int b = 0; b < RJ; ++b) win[a][b] = gr[a * GC + b];
+        // column q0 + v with the window's column b at position (v + b) mod RJ;
+        // the f values of the next RJ columns are loaded ahead
+        float fv[RJ];
+#pragma unroll
+        for (int v = 0; v < RJ; ++v) fv[v] = fr[v];
+        auto column = [&](int q0, int v) {
+            const float x = fv[v];
+            fv[v] = fr[q0 + v + RJ];                              // (past the row at its end: not used)
+#pragma unroll
+            for (int a = 0; a < RI; ++a) {
+#pragma unroll
+                for (int b = 0; b < RJ; ++b) acc[a][b] = fmaf(x, win[a][(v + b) % RJ], acc[a][b]);
+                win[a][v] = gr[a * GC + q0 + v + RJ];
             }
+        };
+#pragma unroll 1
+        for (int q0 = 0; q0 + RJ <= kMapCols; q0 += RJ)
+#pragma unroll
+            for (int v = 0; v < RJ; ++v) column(q0, v);
+#pragma unroll
+        for (int v = 0; v < kMapCols % RJ; ++v) column(kMapCols - kMapCols % RJ, v);
+    }
+    const int64_t nshift = (int64_t)ndi * ndj, nchunks = (int64_t)nrc * ncc;
+    float* o = part + ((int64_t)pc * nchunks + (int64_t)rc * ncc + cc) * nshift;
+#pragma unroll
+    for (int a = 0; a < RI; ++a) {
+        const int di = di_lo + ui * RI + a;
+#pragma unroll
+        for (int b = 0; b < RJ; ++b) {
+            const int dj = dj_lo + uj * RJ + b;
+            if (di <= max_di && dj <= max_dj) o[(int64_t)(di + max_di) * ndj + (dj + max_dj)] = acc[a][b];
         }
     }
 }
@@ -225,7 +280,8 @@ __global__ void __launch_bounds__(256) xmap_sum(const float* __restrict__ part, 
     colsum[t] = (double)sum - (double)comp;
 }
 
-__global__ void __launch_bounds__(256) xmap_finish(const double* __restrict__ colsum,
+// (one warp a block: the divisions, FP64, spread over the SMs)
+__global__ void __launch_bounds__(32) xmap_finish(const double* __restrict__ colsum,
                                                    const double* __restrict__ stats, int n_pairs, int C, int ncc,
                                                    int nshift, double* __restrict__ out)
 {
@@ -249,44 +305,110 @@ __global__ void __launch_bounds__(256) xmap_finish(const double* __restrict__ co
 }
 
 // Peak of the stacked-channel map: largest value, the first in row-major
-// order (di, then dj ascending) among equal ones.
+// order (di, then dj ascending) among equal ones.  Values are compared as
+// integers of the same order (FP64 compares run on the FP64 pipe); NaN is
+// below all.
+__device__ __forceinline__ long long xmap_key(double v)
+{
+    const long long u = __double_as_longlong(v);
+    const long long k = u >= 0 ? u : (long long)0x8000000000000000ull - u;      // -0.0 as 0.0
+    return v == v ? k : (long long)0x8000000000000000ull;
+}
+
 __global__ void __launch_bounds__(1024) xmap_peak(const double* __restrict__ map, int C, int max_di, int max_dj,
                                                   double* __restrict__ peak)
 {
     const int ndj = 2 * max_dj + 1, nshift = (2 * max_di + 1) * ndj;
-    double best = -INFINITY;
+    long long best = (long long)0x8000000000000000ull;
     int bi = nshift;
     for (int s = threadIdx.x; s < nshift; s += blockDim.x) {
-        const double v = map[(int64_t)s * (C + 1) + C];
-        if (v > best || (v == best && s < bi)) { best = v; bi = s; }
+        const long long v = xmap_key(map[(int64_t)s * (C + 1) + C]);
+        if (v > best) { best = v; bi = s; }
     }
-    __shared__ double sv[32];
+    __shared__ long long sv[32];
     __shared__ int si[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_down_sync(0xffffffffu, best, o);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-    }
+    auto reduce = [&]() {
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long ov = __shfl_down_sync(0xffffffffu, best, o);
+            const int oi = __shfl_down_sync(0xffffffffu, bi, o);
+            if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+        }
+    };
+    reduce();
     if (lane == 0) { sv[warp] = best; si[warp] = bi; }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-            if (sv[w] > best || (sv[w] == best && si[w] < bi)) { best = sv[w]; bi = si[w]; }
-        peak[0] = best;
-        peak[1] = (double)(bi / ndj - max_di);
-        peak[2] = (double)(bi % ndj - max_dj);
+    if (warp == 0) {
+        best = sv[lane];
+        bi = si[lane];
+        reduce();
+        if (lane == 0) {
+            peak[0] = bi < nshift ? map[(int64_t)bi * (C + 1) + C] : -INFINITY;
+            peak[1] = (double)(bi / ndj - max_di);
+            peak[2] = (double)(bi % ndj - max_dj);
+        }
     }
 }
 
-template <int R>
-static cudaError_t launch_tiles(dim3 grid, cudaStream_t st, const MapImages& im, const double* stats, int H, int W,
-                               int C, int j0, int j1, int max_di, int max_dj, int ncc, int nchunks, float* part)
+// Layout of the tiles for ri x rj shifts a thread.
+static MapPlan map_plan(int ri, int rj, int ndi, int ndj, int nrc)
 {
-    const size_t smem = MapTile<R>::smem;
-    cudaError_t e = cudaFuncSetAttribute(xmap_tiles<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    MapPlan p;
+    p.ri = ri;
+    p.rj = rj;
+    p.gi = (ndi + ri - 1) / ri;
+    p.gj = (ndj + rj - 1) / rj;
+    const int tiles = (p.gi * p.gj + kMapThreads - 1) / kMapThreads;
+    p.git = (p.gi + tiles - 1) / tiles;
+    while (p.git * p.gj > kMapThreads) --p.git;
+    p.kc = std::max(1, std::min(std::min(nrc, 8), kMapThreads / (p.git * p.gj)));
+    // row length of the window: ri gc = 1 (mod 32) puts the lanes of different
+    // di groups on banks one apart, between those of the dj groups (rj apart)
+    p.gc = kMapCols + p.gj * rj + 1;
+    while ((ri * p.gc) % 32 != 1) ++p.gc;
+    auto bytes = [&] {
+        return sizeof(float) * ((size_t)(p.kc * kMapRows + p.git * ri - 1) * p.gc + (size_t)p.kc * kMapRows * kMapCols + 16);
+    };
+    while (p.kc > 1 && bytes() > (size_t)74 * 1024) --p.kc;        // three blocks per SM
+    p.smem = bytes();
+    // few shifts keep few threads busy, but the block's window wants loading
+    p.threads = std::max(128, (p.kc * p.git * p.gj + 31) / 32 * 32);
+    return p;
+}
+
+// The shifts a thread owns: few enough that the launch fills the chip, many
+// enough to load little.  The cost is the blocks of the fullest SM times a
+// block's warps on its scheduler times the cycles of a column (FMAs and loads
+// to issue, or the SM's shared memory delivering one load a cycle to four
+// schedulers), and the block's loads.
+static MapPlan choose_plan(int ndi, int ndj, int nrc, int ncc, int npc)
+{
+    constexpr int kSMs = 152;
+    MapPlan best = {};
+    double least = 1e300;
+    for (int ri : {1, 3})
+        for (int rj : {3, 5, 9, 13}) {
+            const MapPlan p = map_plan(ri, rj, ndi, ndj, nrc);
+            const int64_t blocks = (int64_t)((p.gi + p.git - 1) / p.git) * ((nrc + p.kc - 1) / p.kc) * ncc * npc;
+            const int warps = (p.kc * p.git * p.gj + 31) / 32;
+            const double column = std::max(warps / 4.0 * (ri * rj + ri + 1), (double)std::max(warps, 4) * (ri + 1));
+            const double load = (double)p.smem / (4.0 * p.threads) * 60.0;
+            const double cost = (double)((blocks + kSMs - 1) / kSMs) * (column * kMapRows * kMapCols + load);
+            if (cost < least) { least = cost; best = p; }
+        }
+    return best;
+}
+
+template <int RI, int RJ>
+static cudaError_t launch_tiles(cudaStream_t st, const MapPlan& p, const MapImages& im, const double* stats, int H,
+                               int W, int C, int j0, int j1, int max_di, int max_dj, int nrc, int ncc, int npc,
+                               float* part)
+{
+    if (p.ri != RI || p.rj != RJ) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(xmap_tiles<RI, RJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return e;
-    xmap_tiles<R><<<grid, kMapBlock, smem, st>>>(im, stats, H, W, C, j0, j1, max_di, max_dj, ncc, nchunks, part);
+    const dim3 grid((unsigned)(((p.gi + p.git - 1) / p.git) * ((nrc + p.kc - 1) / p.kc) * ncc), npc);
+    xmap_tiles<RI, RJ><<<grid, p.threads, p.smem, st>>>(im, stats, H, W, C, j0, j1, max_di, max_dj, nrc, ncc, p, part);
     return cudaGetLastError();
 }
 
@@ -336,9 +458,9 @@ extern "C" int rt_xcorr_map(const float* const* d_f, const float* const* d_g, in
                                          sizeof(double) * (size_t)n_pairs * mchunks * channels * 3) + 255) &
                                ~(size_t)255;
     const size_t ncol = (size_t)npc * ncc * nshift;
-    const size_t part_bytes = chunk_bytes + sizeof(double) * ncol;
-    cudaError_t e = scratch_alloc((void**)&stats, sizeof(double) * 3 * npc, st);
-    if (e == cudaSuccess) e = scratch_alloc((void**)&partial, part_bytes, st);
+    const size_t part_bytes = chunk_bytes + sizeof(double) * (ncol + 3 * (size_t)npc);
+    cudaError_t e = scratch_alloc((void**)&partial, part_bytes, st);
+    if (e == cudaSuccess) stats = (double*)((char*)partial + chunk_bytes) + ncol;
     if (e == cudaSuccess) {
         xmap_moment_rows<<<dim3(mchunks, n_pairs), kMomBlock, 0, st>>>(im, height, width, channels, j0, j1, mchunks,
                                                                         partial);
@@ -349,23 +471,14 @@ extern "C" int rt_xcorr_map(const float* const* d_f, const float* const* d_g, in
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        // shifts per thread along each axis: the smallest odd R with
-        // 16 R >= the larger shift range (1, 3 or 5; ranges past 80 take
-        // more tiles of R = 5)
-        const int nd = std::max(ndi, ndj);
-        const int R = nd <= kMapT ? 1 : (nd <= 3 * kMapT ? 3 : 5);
-        const int TD = kMapT * R;
-        const dim3 grid(((ndi + TD - 1) / TD) * ((ndj + TD - 1) / TD), nchunks, npc);
+        const MapPlan p = choose_plan(ndi, ndj, nrc, ncc, npc);
         float* part = (float*)partial;
-        if (R == 1)
-            e = launch_tiles<1>(grid, st, im, stats, height, width, channels, j0, j1, max_di, max_dj, ncc, nchunks,
-                                part);
-        else if (R == 3)
-            e = launch_tiles<3>(grid, st, im, stats, height, width, channels, j0, j1, max_di, max_dj, ncc, nchunks,
-                                part);
-        else
-            e = launch_tiles<5>(grid, st, im, stats, height, width, channels, j0, j1, max_di, max_dj, ncc, nchunks,
-                                part);
+#define RT_TILES(RI, RJ)                                                                                              \
+    if (e == cudaSuccess)                                                                                             \
+        e = launch_tiles<RI, RJ>(st, p, im, stats, height, width, channels, j0, j1, max_di, max_dj, nrc, ncc, npc, part)
+        RT_TILES(1, 3); RT_TILES(1, 5); RT_TILES(1, 9); RT_TILES(1, 13);
+        RT_TILES(3, 3); RT_TILES(3, 5); RT_TILES(3, 9); RT_TILES(3, 13);
+#undef RT_TILES
     }
     double* colsum = partial ? (double*)((char*)partial + chunk_bytes) : nullptr;
     if (e == cudaSuccess) {
@@ -374,7 +487,7 @@ extern "C" int rt_xcorr_map(const float* const* d_f, const float* const* d_g, in
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        xmap_finish<<<(nshift + 255) / 256, 256, 0, st>>>(colsum, stats, n_pairs, channels, ncc, nshift, d_map);
+        xmap_finish<<<(nshift + 31) / 32, 32, 0, st>>>(colsum, stats, n_pairs, channels, ncc, nshift, d_map);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && d_peak) {
@@ -382,7 +495,6 @@ extern "C" int rt_xcorr_map(const float* const* d_f, const float* const* d_g, in
         e = cudaGetLastError();
     }
     if (partial) cudaFreeAsync(partial, st);
-    if (stats) cudaFreeAsync(stats, st);
     if (e != cudaSuccess) {
         set_error("rt_xcorr_map: %s", cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? RT_ENOMEM : RT_ECUDA;
