@@ -47,8 +47,8 @@ inline int default_min_active(int precision, int mode)
 constexpr int kMaxWindows = 16;
 // Render mode: the integrator (RT_RK4, RT_DP45, RT_RK4T), with kModeGauss set
 // for scenes of the Gaussian bump, whose box holds the Gaussian map's medium.
-// kModeSplit: FP64 RK4 in the grating cloak with the step of rt_split.cuh, for
-// scenes within its bounds (SplitConst::ok); wavefront loop only.
+// kModeSplit: FP64 RK4 or Dormand-Prince in the grating cloak with the steps of
+// rt_split.cuh, for scenes within their bounds (SplitConst::ok); wavefront loop only.
 constexpr int kModeGauss = 8;
 constexpr int kModeSplit = 16;
 inline int render_mode(const rt_scene_desc& d)
@@ -58,7 +58,7 @@ inline int render_mode(const rt_scene_desc& d)
 // The mode of the wavefront loop a scene is rendered with.
 inline int wave_mode(int precision, int mode, const DevScene& sc)
 {
-    return precision == RT_FP64 && mode == RT_RK4 && sc.sp.ok ? mode | kModeSplit : mode;
+    return precision == RT_FP64 && (mode == RT_RK4 || mode == RT_DP45) && sc.sp.ok ? mode | kModeSplit : mode;
 }
 // Coefficients of the Faddeeva series of the Gaussian cloak, uploaded once
 // per device before its first Gaussian scene.

@@ -38,12 +38,12 @@ static cudaError_t wave_prepare()
 template <class R, int INTEG>
 static cudaError_t occupancy_t(int variant, bool opt, int* bps)
 {
-    if constexpr (split_of(INTEG)) {
+    if constexpr ((INTEG & kModeSplit) != 0) {
         // the wavefront loop only: the per-lane loop steps in FP64
         if (variant != kVariantWave) return occupancy_t<R, (INTEG & ~kModeSplit)>(variant, opt, bps);
     }
     if (variant == kVariantWave) {
-        if constexpr (!gauss_of(INTEG) && !split_of(INTEG)) {
+        if constexpr (!gauss_of(INTEG) && !(INTEG & kModeSplit)) {
             if (opt) {
                 const cudaError_t e = wave_prepare<R, INTEG, true>();
                 if (e != cudaSuccess) return e;
@@ -57,7 +57,7 @@ static cudaError_t occupancy_t(int variant, bool opt, int* bps)
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, wave_kernel<R, INTEG, false>,
                                                              WaveShape<R, INTEG>::kBlock, wave_smem_bytes<R, INTEG>());
     }
-    if constexpr (integ_of(INTEG) == RT_RK4T || gauss_of(INTEG) || split_of(INTEG)) {
+    if constexpr (integ_of(INTEG) == RT_RK4T || gauss_of(INTEG) || (INTEG & kModeSplit)) {
         return cudaErrorInvalidValue;                // the wavefront loop only
     } else {
     if constexpr (sizeof(R) == 4 && INTEG == RT_RK4) {
@@ -78,7 +78,7 @@ static cudaError_t launch_t(const DevScene& sc, int variant, int min_active, flo
     if (variant == kVariantWave) {
         // scenes with options (RT_FLAG_*) take the options build of the loop;
         // the Gaussian bump has none
-        if constexpr (!gauss_of(INTEG) && !split_of(INTEG)) {
+        if constexpr (!gauss_of(INTEG) && !(INTEG & kModeSplit)) {
             if (sc.flags) {
                 const cudaError_t e = wave_prepare<R, INTEG, true>();
                 if (e != cudaSuccess) return e;
@@ -93,7 +93,7 @@ static cudaError_t launch_t(const DevScene& sc, int variant, int min_active, flo
             sc, rgb, rgb8, rec, counters, min_active, ss.col, ss.cnt, ss.br, WaveWait{wl.spin, wl.hold});
         return cudaGetLastError();
     }
-    if constexpr (integ_of(INTEG) == RT_RK4T || gauss_of(INTEG) || split_of(INTEG)) {
+    if constexpr (integ_of(INTEG) == RT_RK4T || gauss_of(INTEG) || (INTEG & kModeSplit)) {
         return cudaErrorInvalidValue;
     } else {
     if constexpr (sizeof(R) == 4 && INTEG == RT_RK4) {
@@ -180,6 +180,7 @@ cudaError_t render_occupancy(int precision, int integrator, int variant, bool op
             case RT_DP45: return occupancy_t<double, RT_DP45>(variant, opt, blocks_per_sm);
             case RT_RK4T: return occupancy_t<double, RT_RK4T>(variant, opt, blocks_per_sm);
             case RT_RK4 | kModeSplit: return occupancy_t<double, RT_RK4 | kModeSplit>(variant, false, blocks_per_sm);
+            case RT_DP45 | kModeSplit: return occupancy_t<double, RT_DP45 | kModeSplit>(variant, false, blocks_per_sm);
             case RT_RK4 | G: return occupancy_t<double, RT_RK4 | G>(variant, false, blocks_per_sm);
             case RT_DP45 | G: return occupancy_t<double, RT_DP45 | G>(variant, false, blocks_per_sm);
             default: return occupancy_t<double, RT_RK4>(variant, opt, blocks_per_sm);
@@ -207,6 +208,7 @@ cudaError_t launch_render(const DevScene& sc, int precision, int variant, int mi
             case RT_DP45: RT_LAUNCH(double, RT_DP45);
             case RT_RK4T: RT_LAUNCH(double, RT_RK4T);
             case RT_RK4 | kModeSplit: RT_LAUNCH(double, RT_RK4 | kModeSplit);
+            case RT_DP45 | kModeSplit: RT_LAUNCH(double, RT_DP45 | kModeSplit);
             case RT_RK4 | G: RT_LAUNCH(double, RT_RK4 | G);
             case RT_DP45 | G: RT_LAUNCH(double, RT_DP45 | G);
             default: RT_LAUNCH(double, RT_RK4);

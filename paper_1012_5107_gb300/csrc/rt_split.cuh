@@ -67,11 +67,20 @@ GRT_HD float frcp(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+GRT_HD float fex2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+GRT_HD void fsincos(float x, float& s, float& c) { __sincosf(x, &s, &c); }
 #else
 GRT_HD float fadd(float a, float b) { return a + b; }
 GRT_HD float fmul(float a, float b) { return a * b; }
 GRT_HD float ffma(float a, float b, float c) { return fmaf(a, b, c); }
 GRT_HD float frcp(float x) { return 1.0f / x; }
+GRT_HD float fex2(float x) { return exp2f(x); }
+GRT_HD void fsincos(float x, float& s, float& c) { s = sinf(x); c = cosf(x); }
 #endif
 GRT_HD float fsub(float a, float b) { return fadd(a, -b); }
 // ... and on pairs, two operations in one instruction (FADD2, FFMA2)
@@ -206,6 +215,13 @@ GRT_HD Z3 split3(double x, double y)
     const F3 a = split3(x), b = split3(y);
     return {float2{a.h, b.h}, float2{a.m, b.m}, float2{a.l, b.l}};
 }
+GRT_HD Z2 split2(double x, double y)
+{
+    const float a = (float)x, b = (float)y;
+    return {float2{a, b}, float2{(float)(x - (double)a), (float)(y - (double)b)}};
+}
+GRT_HD double join_x(Z2 a) { return (double)a.h.x + (double)a.l.x; }
+GRT_HD double join_y(Z2 a) { return (double)a.h.y + (double)a.l.y; }
 GRT_HD double join_x(Z3 a) { return (double)a.h.x + ((double)a.m.x + (double)a.l.x); }
 GRT_HD double join_y(Z3 a) { return (double)a.h.y + ((double)a.m.y + (double)a.l.y); }
 
@@ -281,21 +297,16 @@ GRT_HD float2 split_guess(float2 v, float2 r, float2 s)
     return cfma(float2{-b.x, -b.y}, t, t);
 }
 
-// Full solve: base W_b with v = W_b/(1 + W_b) and r = 1/(1 + W_b) in FP32,
-// displacement s.  Returns P = W_b (exp(d) - 1), so that W = W_b + P, and W.
-GRT_HD void split_solve(Z2 wb, float2 v, float2 r, Z2 s, Z2& p, Z2& w)
+// Newton step of the solve at d0 = z with E = exp(z) - 1: P = W_b E and the
+// residual s - z - P, then P and W = W_b + P with the step taken.
+GRT_HD void split_newton(Z2 wb, float2 z, Z2 e, Z2 s, Z2& p, Z2& w)
 {
-    const float2 z = split_guess(v, r, s.h);
-    // residual R = s - d0 - W_b (exp(d0) - 1): the leading parts nearly cancel,
-    // their remainders are of its size
-    Z2 e = split_expm1_tail(z);
-    const Z2 e1 = two_sum(z, e.h);
-    e = {e1.h, vadd(e1.l, e.l)};
+    // the leading parts nearly cancel, their remainders are of the residual's size
     p = zmulu(wb, e);
     const Z2 r1 = two_sum(s.h, vneg(z)), r2 = two_sum(r1.h, vneg(p.h));
     const Z2 R = {r2.h, vadd(vadd(r1.l, r2.l), vsub(s.l, p.l))};
-    // Newton step D = R/(1 + W1), W1 = W_b exp(d0): an FP32 reciprocal q,
-    // corrected by c = 1 - q (1 + W1), whose leading parts cancel exactly
+    // D = R/(1 + W1), W1 = W_b exp(z): an FP32 reciprocal q, corrected by
+    // c = 1 - q (1 + W1), whose leading parts cancel exactly
     const Z2 w1 = add(wb, p);
     const F2 a1 = fast_two_sum(1.0f, w1.h.x);
     const float ax = a1.h, ay = w1.h.y, bx = fadd(a1.l, w1.l.x), by = w1.l.y;
@@ -305,13 +316,52 @@ GRT_HD void split_solve(Z2 wb, float2 v, float2 r, Z2 s, Z2& p, Z2& w)
     const float2 c = {ffma(q.y, by, ffma(-q.x, bx, fsub(ffma(q.y, ay, fsub(1.0f, c1.h)), c1.l))),
                       -ffma(q.y, bx, ffma(q.x, by, fadd(ffma(q.y, ax, c2.h), c2.l)))};
     Z2 d = zmulf(R, q);
-    // exp(d) - exp(d0) = exp(d0) (D + D^2 q/2): the second order of both the
-    // root and the exponential
+    // exp(d) - exp(z) = exp(z) (D + D^2 q/2): the second order of both the root
+    // and the exponential
     const float2 g = cfma(d.h, float2{0.5f * q.x, 0.5f * q.y}, c);
     d.l = vadd(d.l, cmul(d.h, g));
     const Z2 wd = zmulu(w1, d);
     p = fast_addu(p, wd);
     w = fast_addu(w1, wd);
+}
+
+// Full solve: base W_b with v = W_b/(1 + W_b) and r = 1/(1 + W_b) in FP32,
+// displacement s.  Returns P = W_b (exp(d) - 1), so that W = W_b + P, and W.
+GRT_HD void split_solve(Z2 wb, float2 v, float2 r, Z2 s, Z2& p, Z2& w)
+{
+    const float2 z = split_guess(v, r, s.h);
+    const Z2 e = split_expm1_tail(z), e1 = two_sum(z, e.h);
+    split_newton(wb, z, Z2{e1.h, vadd(e1.l, e.l)}, s, p, w);
+}
+
+// The solve for |s| up to 0.6 (Dormand-Prince stages), from the FP32 guess z,
+// which Newton steps in FP32 improve and leave in z: exp(z) - 1 from z/8, by
+// E <- 2 E + E^2 three times.  Returns P.
+GRT_HD Z2 split_solve_wide(Z2 wb, Z2 s, float2& z)
+{
+    for (int it = 0; it < 8; ++it) {
+        const float m = fex2(fmul(z.x, 1.44269504f));
+        float sn, cs;
+        fsincos(z.y, sn, cs);
+        const float2 E = {ffma(m, cs, -1.0f), fmul(m, sn)};
+        const float2 u = cmul(wb.h, E);
+        const float2 R = {fsub(fsub(s.h.x, z.x), u.x), fsub(fsub(s.h.y, z.y), u.y)};
+        const float ax = fadd(1.0f + wb.h.x, u.x), ay = fadd(wb.h.y, u.y);
+        const float inv = frcp(ffma(ax, ax, fmul(ay, ay)));
+        const float2 d = {fmul(ffma(R.x, ax, fmul(R.y, ay)), inv), fmul(ffma(R.y, ax, -fmul(R.x, ay)), inv)};
+        z = vadd(z, d);
+        if (!(ffma(d.x, d.x, fmul(d.y, d.y)) > 1e-8f)) break;      // the next step would be 1e-8 at most
+    }
+    const float2 x = {0.125f * z.x, 0.125f * z.y};
+    const Z2 t = split_expm1_tail(x), e1 = two_sum(x, t.h);
+    Z2 e = {e1.h, vadd(e1.l, t.l)};
+#if defined(__CUDACC__)
+#pragma unroll 1
+#endif
+    for (int q = 0; q < 3; ++q) e = add(scale(e, 2.0f), zmulu(e, e));
+    Z2 p, w;
+    split_newton(wb, z, e, s, p, w);
+    return p;
 }
 
 // Continuation over a small s (|s| <= 1e-3) from a point whose W and r are

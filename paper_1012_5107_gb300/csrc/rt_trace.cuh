@@ -52,7 +52,9 @@ __host__ __device__ constexpr int integ_of(int mode) { return mode & 7; }
 __host__ __device__ constexpr bool gauss_of(int mode) { return (mode & kModeGauss) != 0; }
 // kModeSplit: the integration loop steps a SplitBox (rt_split.cuh) instead of
 // a Box<double>; the service code is the FP64 path's.
-__host__ __device__ constexpr bool split_of(int mode) { return (mode & kModeSplit) != 0; }
+__host__ __device__ constexpr bool split_of(int mode) { return (mode & kModeSplit) != 0 && integ_of(mode) == RT_RK4; }
+// ... and with Dormand-Prince the FP64 state's stages in two floats (dp45_step_wide).
+__host__ __device__ constexpr bool wide_of(int mode) { return (mode & kModeSplit) != 0 && integ_of(mode) == RT_DP45; }
 
 enum : int { PH_IDLE = 0, PH_AIR = 1, PH_BOX = 2, PH_DONE = 3, PH_EXIT = 4, PH_EVENT = 5, PH_GUARD = 6 };
 enum : int { EV_NONE = -1, EV_GRATING = 0, EV_TOP = 1, EV_XP = 2, EV_XM = 3, EV_ZP = 4, EV_ZM = 5, EV_COUNT = 6 };
@@ -821,6 +823,81 @@ __device__ __forceinline__ void dp45_step_sums(const StepConst<R>& k, const Box<
     wrap_cell<R, INTEG>(o);
 }
 
+// The FP64 step with W0 at its stages carried from the step's start in two
+// floats (split_solve_wide): a carried W0 is good to 1e-14 of its change over the
+// step, which enters the force, and the force the state, scaled by the step.
+// The forces, their sums, whose coefficients reach 10 and cancel, and the state
+// stay FP64 (with the forces or their sums in two floats the exits' rounding was
+// three times the FP64 step's), and W0 at the end takes one FP64 Newton step, so
+// nothing is carried from step to step in less than FP64.  The library
+// exponentials and sine/cosines of the stages' solves were most of the step's
+// 1,200 FP64 instructions; some 480 are left.
+template <int INTEG>
+__device__ __forceinline__ void dp45_step_wide(const StepConst<double>& k, const Box<double>& s, double h, Box<double>& o,
+                                               double e[4], LaneStats& st)
+{
+    const Z2 wb = split2(s.wr, s.wi);
+    float2 z = {0.0f, 0.0f}, dp = z, r = {(float)s.rr, (float)s.ri};
+    const double hpx = h * s.px, hpy = h * s.py, hh = h * h;
+    double Fx[7], Fy[7];
+    Fx[0] = s.Fx;
+    Fy[0] = s.Fy;
+    double dx = 0.0, dy = 0.0, wr = s.wr, wi = s.wi;
+#pragma unroll 1
+    for (int j = 2; j <= 7; ++j) {
+        double ax = 0.0, ay = 0.0;
+        const int nl = (j < 7) ? j - 2 : 6;
+#pragma unroll 1
+        for (int l = 0; l < nl; ++l) {
+            const double a = dp_tab_aa<double>(j - 2, l);
+            ax += a * Fx[l];
+            ay += a * Fy[l];
+        }
+        dx = dp_tab_c<double>(j - 2) * hpx + hh * ax;
+        dy = dp_tab_c<double>(j - 2) * hpy + hh * ay;
+        const Z2 d = split2(-kTwoPi * dy, kTwoPi * dx);
+        // the previous stage's solution moved on by r (D - D_prev)
+        z = cfma(vsub(d.h, dp), r, z);
+        dp = d.h;
+        const Z2 p = split_solve_wide(wb, d, z);
+        wr = s.wr + join_x(p);
+        wi = s.wi + join_y(p);
+        const double ar = 1.0 + wr, inv = recip_nr(ar * ar + wi * wi), rr = ar * inv, ri = -wi * inv;
+        r = float2{(float)rr, (float)ri};
+        ray_force(wr, wi, rr, ri, k.fk, Fx[j - 1], Fy[j - 1]);
+    }
+    double fx = 0.0, fy = 0.0, ex = 0.0, ey = 0.0, gx = 0.0, gy = 0.0;
+#pragma unroll
+    for (int l = 1; l <= 7; ++l) {
+        if (l <= 6) {
+            fx += dp_a(7, l) * Fx[l - 1];
+            fy += dp_a(7, l) * Fy[l - 1];
+            ex += dp_ea(l) * Fx[l - 1];
+            ey += dp_ea(l) * Fy[l - 1];
+        }
+        gx += dp_e(l) * Fx[l - 1];
+        gy += dp_e(l) * Fy[l - 1];
+    }
+    o = s;
+    o.X = s.X + dx;
+    o.y = s.y + dy;
+    o.z = s.z + h * s.pz;
+    o.px = s.px + h * fx;
+    o.py = s.py + h * fy;
+    e[0] = hh * ex;
+    e[1] = hh * ey;
+    e[2] = h * gx;
+    e[3] = h * gy;
+    o.wr = wr;
+    o.wi = wi;
+    double dr, di;
+    newton_w0(k.kA, o.X, o.y, o.wr, o.wi, o.rr, o.ri, dr, di);
+    ray_force(o.wr, o.wi, o.rr, o.ri, k.fk, o.Fx, o.Fy);
+    st.evals += 6;
+    st.newton += 13;
+    wrap_cell<double, INTEG>(o);
+}
+
 // FP32 takes the running sums (13 % faster on the 1920 x 1080 workload);
 // FP64 the table, since the sums' 24 more registers cost it occupancy (4 %
 // slower).
@@ -830,6 +907,8 @@ __device__ __forceinline__ void dp45_step(const StepConst<R>& k, const Box<R>& s
 {
     if constexpr (sizeof(R) == 4)
         dp45_step_sums<R, INTEG>(k, s, h, o, e, st);
+    else if constexpr (wide_of(INTEG))
+        dp45_step_wide<INTEG>(k, s, h, o, e, st);
     else
         dp45_step_table<R, INTEG>(k, s, h, o, e, st);
 }
@@ -957,7 +1036,7 @@ __device__ __forceinline__ void face_normal(int ev, R N[3])
 template <class R, int INTEG>
 __host__ __device__ constexpr bool resolve_end()
 {
-    return !(sizeof(R) == 4 && integ_of(INTEG) == RT_DP45) && !split_of(INTEG);
+    return !(sizeof(R) == 4 && integ_of(INTEG) == RT_DP45) && !split_of(INTEG) && !wide_of(INTEG);
 }
 
 // Root theta in (0, 1] of g_ev(Phi_{theta h}(b)) given its value g1 < 0 at
@@ -1863,6 +1942,17 @@ __device__ __forceinline__ void box_step_into(const StepConst<R>& k, int64_t max
             const R err2 = R(0.25) * (q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3);
             err = err2;                                                   // err <= 1 iff err^2 <= 1
             fac = (err2 > R(0)) ? R(0.9) * Mth<R>::ex2(R(-0.1) * Mth<R>::lg2(err2)) : R(5);
+        } else if constexpr (wide_of(INTEG)) {
+            // the same to 1e-13: refined reciprocals, and err^-1/5 = (err^2)^-1/10
+            // from an FP32 seed y by y (1 + c/10 + 11 c^2/200), c = 1 - err^2 y^10
+            const R ip = recip_nr(scp), q0 = e[0] * ip, q1 = e[1] * ip, q2 = e[2] * recip_nr(s2), q3 = e[3] * recip_nr(s3);
+            err = R(0.25) * (q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3);      // err <= 1 iff err^2 <= 1
+            fac = R(5);
+            if (err > R(1e-30)) {
+                const R y = (R)Mth<float>::ex2(-0.1f * Mth<float>::lg2((float)fmin(err, R(1e30))));
+                const R y2 = y * y, y4 = y2 * y2, c = fma(-err, y4 * y4 * y2, R(1));
+                fac = R(0.9) * (y * fma(c, fma(c, R(0.055), R(0.1)), R(1)));
+            }
         } else {
             const R q0 = e[0] / scp, q1 = e[1] / scp, q2 = e[2] / s2, q3 = e[3] / s3;
             err = Mth<R>::sqrt_(R(0.25) * (q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3));

@@ -71,3 +71,38 @@ def test_split_render_repeats_and_matches_for_every_grouping():
         sc.render(rgb, rec=rec)
         out.append(rec.cpu().numpy())
     assert all(np.array_equal(out[0], o) for o in out[1:])
+
+
+# Dormand-Prince: the steps' sizes follow the error estimates, whose rounding is
+# 1e-10 of them on both sides, so the two sides' exits differ by 1e-10 of the
+# tolerance (1e-7) and by their rounding; the bar is again 1e-10.
+@pytest.mark.parametrize("over", [
+    dict(),
+    dict(A=0.0),
+    dict(A=0.0477),
+    dict(A=0.048, width=24, height=20),                 # past kA = 0.3: the general step
+    dict(rtol=1e-3, atol=1e-3),                         # steps of h_max: the general step
+    dict(rtol=1e-6, atol=1e-6, A=0.01),                 # the loosest tolerance, weak forces: the longest steps
+    dict(rtol=1e-10, atol=1e-10, width=20, height=16),
+    dict(h_max=1.0 / 15.0, A=0.04),                     # |D| = 0.56 at n_max: the general step
+    dict(h=0.5, h_max=0.06),                            # a first step past the bound: the general step
+    dict(H=7.9, E=24.0, cam_dist=30.0, width=24, height=20),
+    dict(H=0.11, E=6.0),
+    dict(E=0.7, elev_deg=12.0),
+    dict(max_steps=12),
+    dict(azim_deg=90.0, elev_deg=15.0),
+    dict(width=7, height=5, spp=3, Lambda=0.6, A=0.02, E=4.8, H=1.2, h=0.003, h_max=0.0375, cam_dist=7.2, bg_cell=0.3),
+])
+def test_wide_stages_equal_general_step(over):
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    p = inputs.base_scene(**{**dict(width=40, height=32, spp=1, precision=1, integrator=inputs.DP45, rtol=1e-7, atol=1e-7),
+                             **over})
+    a_rgb, a, a_st = render(rt, torch, p, 0)
+    b_rgb, b, b_st = render(rt, torch, p, 3)
+    assert a_st["rays"] == b_st["rays"] and a_st["steps"] == b_st["steps"] and a_st["status"] == b_st["status"]
+    for name in ("status", "bounces", "events", "steps"):
+        assert np.array_equal(a[name], b[name]), name
+    assert np.abs(a["pos"] - b["pos"]).max() <= 1e-10 * p["Lambda"]
+    assert np.abs(a["dir"] - b["dir"]).max() <= 1e-10
+    assert np.array_equal(a_rgb, b_rgb)
