@@ -31,14 +31,18 @@ constexpr int kMinActiveRK4F32 = 24;
 constexpr int kMinActiveF64 = 32;
 constexpr int kMinActiveSplit = 28;
 // Dormand-Prince steps are longer: a task holding fewer rays is still worth
-// running (1920 x 1080 x 16 with one block of 384 threads per SM, E = 8 / 32:
-// 133.0 / 214.8 ms at 8, 135.1 / 221.5 ms at 16; 2 to 10 within 1 %)
+// running (1920 x 1080 x 16, E = 8 / 32: 113.7 / 202.0 ms at 4, 113.3 / 207.4
+// at 8, 111.7 / 218.0 at 16); the Gaussian and FP64 builds at 8, the FP64 build
+// with stages in two floats at 24 (128 x 128 x 4: 6.99 ms, 7.44 at 8)
 constexpr int kMinActiveDP45 = 8;
+constexpr int kMinActiveDP45F32 = 4;
+constexpr int kMinActiveWide = 24;
 // The default for a precision (RT_FP32 / RT_FP64) and render mode (the
 // integrator, with kModeGauss for the Gaussian bump).
 inline int default_min_active(int precision, int mode)
 {
-    if ((mode & 7) == RT_DP45) return kMinActiveDP45;
+    if ((mode & 7) == RT_DP45)
+        return (mode & 16) ? kMinActiveWide : precision == RT_FP32 && mode == RT_DP45 ? kMinActiveDP45F32 : kMinActiveDP45;
     if (mode & 16) return kMinActiveSplit;
     if (precision == RT_FP64) return kMinActiveF64;
     if (mode == RT_RK4) return kMinActiveRK4F32;
@@ -147,7 +151,8 @@ namespace grt {
 bool tune_lookup(const std::string& key, int* variant, int* min_active);
 // Scene table of a validated descriptor (texture pointer left to the caller).
 void build_scene_table(const rt_scene_desc* d, DevScene* s);
-cudaError_t batch_occupancy(int precision, int integrator, bool opt, int* bps);
+// `mode`: the integrator, with kModeSplit where every cloaked scene takes it.
+cudaError_t batch_occupancy(int precision, int mode, bool opt, int* bps);
 // One launch of the wavefront loop over the pixels of n scenes (device tables).
 struct BatchLaunch {
     const DevScene* scenes;
@@ -161,7 +166,7 @@ struct BatchLaunch {
     int min_active, grid;
     bool opt;                    // a scene has options (RT_FLAG_*): the options build
 };
-cudaError_t launch_batch(int precision, int integrator, const BatchLaunch& L, cudaStream_t stream);
+cudaError_t launch_batch(int precision, int mode, const BatchLaunch& L, cudaStream_t stream);
 void tune_record(const std::string& key, int variant, int min_active);
 
 }  // namespace grt

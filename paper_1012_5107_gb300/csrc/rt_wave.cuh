@@ -44,13 +44,21 @@ constexpr int kWaveSpin = kDefaultWaitSpin;  // attempts (with a short sleep) be
 // block, blocks per SM (which sets the registers a thread may use: 65536 /
 // (threads x blocks)) and P, the samples in flight per block -- more than the
 // block's lanes, so that a warp always finds work while the other warps hold
-// theirs.  FP32 RK4: two blocks of 256 threads, 128 registers.  FP32
+// theirs.  FP32: two blocks of 256 threads, 128 registers.  FP32
 // Dormand-Prince keeps the running sums of its stages and two states live
-// through a step, which spills at 128 registers: one block of 384 threads
-// (12 warps, up to 168 registers).  FP64: one block of 256 threads.
+// through a step, which spills 370 bytes at 128 registers; with the step's
+// start left in the pool (kInPool: it is read at the step's ends only) it
+// spills 290 and 16 warps an SM beat the 12 that 168 registers allow (1920 x
+// 1080 x 16, E = 2 / 8 / 32: 18.4 / 113.7 / 202.0 ms against 20.2 / 115.7 /
+// 204.0 with one block of 384; with the start in registers 19.4 / 125.2 /
+// 230.6).  FP32 RK4 in the pool is slower (7.07 -> 8.57 ms the step's launch:
+// its steps are a quarter as long).  The Gaussian Dormand-Prince keeps the
+// block of 384.  FP64: one block of 256 threads; the split RK4 step two.
 template <class R, int INTEG>
 struct WaveShape {
-    static constexpr bool kWide = sizeof(R) == 4 && integ_of(INTEG) == RT_DP45;
+    static constexpr bool kDp = sizeof(R) == 4 && integ_of(INTEG) == RT_DP45;
+    static constexpr bool kWide = kDp && gauss_of(INTEG);
+    static constexpr bool kInPool = kDp && !gauss_of(INTEG);
     static constexpr int kBlock = kWide ? 384 : 256;
     static constexpr int kMinBlocks = ((sizeof(R) == 4 && !kWide) || split_of(INTEG)) ? 2 : 1;
     static constexpr int P = kWide ? 576 : (sizeof(R) == 4 ? 384 : (split_of(INTEG) ? 280 : 320));
@@ -344,8 +352,9 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
         } else if (task == WT_INT) {
             // ---- integrate ----
             if constexpr (!split_of(INTEG)) {
+            // (kInPool steps the pool's entry in place)
             if (p >= 0) {
-                b = boxes[p];
+                if constexpr (!WaveShape<R, INTEG>::kInPool) b = boxes[p];
                 phase = PH_BOX;
                 surf = C.surf;
                 steps = C.steps;
@@ -365,11 +374,16 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
 #if RT_PROFILE
                 prof[2] += 1;
 #endif
-                if (phase == PH_BOX) box_step<R, INTEG>(*kp, max_steps, C, b, phase, surf, steps, st, safe);
+                if (phase == PH_BOX) {
+                    if constexpr (WaveShape<R, INTEG>::kInPool)
+                        box_step<R, INTEG>(*kp, max_steps, C, boxes[p], phase, surf, steps, st, safe);
+                    else
+                        box_step<R, INTEG>(*kp, max_steps, C, b, phase, surf, steps, st, safe);
+                }
                 if (__popc(__ballot_sync(0xffffffffu, phase == PH_BOX)) < need) break;
             }
             if (p >= 0) {
-                boxes[p] = b;
+                if constexpr (!WaveShape<R, INTEG>::kInPool) boxes[p] = b;
                 C.surf = surf;
                 C.steps = steps;
                 C.phase = phase;
