@@ -45,6 +45,10 @@ static cudaError_t batch_occupancy_t(int* bps)
 template <bool OPT>
 static cudaError_t batch_occupancy_o(int precision, int integrator, int* bps)
 {
+    if constexpr (!OPT) {
+        if (integrator == (RT_RK4 | kModeSplit)) return batch_occupancy_t<double, RT_RK4 | kModeSplit, OPT>(bps);
+        if (integrator == (RT_DP45 | kModeSplit)) return batch_occupancy_t<double, RT_DP45 | kModeSplit, OPT>(bps);
+    }
     if (precision == RT_FP64) {
         if (integrator == RT_DP45) return batch_occupancy_t<double, RT_DP45, OPT>(bps);
         if (integrator == RT_RK4T) return batch_occupancy_t<double, RT_RK4T, OPT>(bps);
@@ -55,10 +59,9 @@ static cudaError_t batch_occupancy_o(int precision, int integrator, int* bps)
     return batch_occupancy_t<float, RT_RK4, OPT>(bps);
 }
 
-cudaError_t batch_occupancy(int precision, int integrator, bool opt, int* bps)
+cudaError_t batch_occupancy(int precision, int mode, bool opt, int* bps)
 {
-    return opt ? batch_occupancy_o<true>(precision, integrator, bps)
-               : batch_occupancy_o<false>(precision, integrator, bps);
+    return opt ? batch_occupancy_o<true>(precision, mode, bps) : batch_occupancy_o<false>(precision, mode, bps);
 }
 
 template <class R, int INTEG, bool OPT>
@@ -75,6 +78,10 @@ static cudaError_t launch_batch_t(const BatchLaunch& L, cudaStream_t stream)
 template <bool OPT>
 static cudaError_t launch_batch_o(int precision, int integrator, const BatchLaunch& L, cudaStream_t stream)
 {
+    if constexpr (!OPT) {
+        if (integrator == (RT_RK4 | kModeSplit)) return launch_batch_t<double, RT_RK4 | kModeSplit, OPT>(L, stream);
+        if (integrator == (RT_DP45 | kModeSplit)) return launch_batch_t<double, RT_DP45 | kModeSplit, OPT>(L, stream);
+    }
     if (precision == RT_FP64) {
         if (integrator == RT_DP45) return launch_batch_t<double, RT_DP45, OPT>(L, stream);
         if (integrator == RT_RK4T) return launch_batch_t<double, RT_RK4T, OPT>(L, stream);
@@ -85,10 +92,9 @@ static cudaError_t launch_batch_o(int precision, int integrator, const BatchLaun
     return launch_batch_t<float, RT_RK4, OPT>(L, stream);
 }
 
-cudaError_t launch_batch(int precision, int integrator, const BatchLaunch& L, cudaStream_t stream)
+cudaError_t launch_batch(int precision, int mode, const BatchLaunch& L, cudaStream_t stream)
 {
-    return L.opt ? launch_batch_o<true>(precision, integrator, L, stream)
-                 : launch_batch_o<false>(precision, integrator, L, stream);
+    return L.opt ? launch_batch_o<true>(precision, mode, L, stream) : launch_batch_o<false>(precision, mode, L, stream);
 }
 
 // ------------------------------------------------------------------------
@@ -166,6 +172,7 @@ using namespace grt;
 
 struct rt_batch {
     int n, device, precision, integrator, grid, nsm, min_active;
+    int mode;                // the integrator, with kModeSplit (batch_mode)
     // The kernel's work list takes the scenes in slot order: slot j holds the
     // caller's scene order[j].  Cloaked scenes (rays that integrate) come
     // first, then bare gratings, then flat mirrors; within a kind the scene
@@ -190,9 +197,23 @@ struct rt_batch {
     unsigned long long* d_counters;
     cudaGraph_t graph;
     cudaGraphExec_t exec;
-    int graph_min_active;
+    int graph_min_active, graph_mode;
     cudaEvent_t done;
 };
+
+// The mode a batch's launch is compiled for: the split double precision steps
+// where every cloaked scene is within their bounds (the others integrate
+// nothing).
+static int batch_mode(int precision, int integrator, bool opt, const std::vector<DevScene>& scenes)
+{
+    bool cloaked = false;
+    for (const DevScene& s : scenes) {
+        if (!s.cloak) continue;
+        cloaked = true;
+        if (wave_mode(precision, integrator, s) == integrator) return integrator;
+    }
+    return cloaked && !opt && precision == RT_FP64 ? integrator | kModeSplit : integrator;
+}
 
 extern "C" {
 
@@ -245,8 +266,9 @@ int rt_batch_create(rt_scene* const* scenes, int32_t n, rt_batch** out)
     b->integrator = integrator;
     b->total = off[n];
     b->total_samples = soff[n];
-    b->min_active = default_min_active(precision, integrator);
-    b->graph_min_active = -1;
+    b->mode = batch_mode(precision, integrator, opt, dev);
+    b->min_active = default_min_active(precision, b->mode);
+    b->graph_min_active = b->graph_mode = -1;
     b->h_rgbs.assign(n, nullptr);
     cudaError_t e = cudaMalloc(&b->d_scenes, sizeof(DevScene) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_offsets, sizeof(int64_t) * (n + 1));
@@ -264,7 +286,7 @@ int rt_batch_create(rt_scene* const* scenes, int32_t n, rt_batch** out)
     int bps = 0;
     b->opt = opt;
     b->h_scenes = dev;
-    if (e == cudaSuccess) e = batch_occupancy(precision, integrator, opt, &bps);
+    if (e == cudaSuccess) e = batch_occupancy(precision, b->mode, opt, &bps);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) {
         set_error("rt_batch_create: %s", cudaGetErrorString(e));
@@ -326,6 +348,13 @@ int rt_batch_update(rt_batch* b, const rt_scene_desc* descs, int32_t n, void* st
         dev[j].pix_list = nullptr;
         dev[j].col_base = old.col_base;
     }
+    const int mode = batch_mode(b->precision, b->integrator, b->opt, dev);
+    if (mode != b->mode) {                      // another kernel: its grid, and the launch recorded again
+        int bps = 0;
+        RT_CK(batch_occupancy(b->precision, mode, b->opt, &bps));
+        b->mode = mode;
+        b->grid = (bps > 0 ? bps : 1) * b->nsm;
+    }
     cudaStream_t st = (cudaStream_t)stream;
     const size_t bytes = sizeof(DevScene) * (size_t)n;
     if (!b->h_stage) {
@@ -355,7 +384,7 @@ int rt_batch_render(rt_batch* b, float* const* d_rgb, void* stream)
         RT_CK(cudaMemcpyAsync(b->d_rgbs, b->h_rgbs.data(), sizeof(float*) * b->n, cudaMemcpyHostToDevice, st));
         RT_CK(cudaStreamSynchronize(st));
     }
-    if (!b->exec || b->graph_min_active != b->min_active) {
+    if (!b->exec || b->graph_min_active != b->min_active || b->graph_mode != b->mode) {
         if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
         if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
         // record the launch (counter reset and the persistent kernel) once
@@ -367,7 +396,7 @@ int rt_batch_render(rt_batch* b, float* const* d_rgb, void* stream)
         const BatchLaunch L = {b->d_scenes, b->d_offsets, b->d_soffsets, b->d_rgbs, b->n, b->total,
                                b->total_samples, {b->d_samp, b->d_pcnt, b->d_br}, b->d_counters, b->min_active,
                                b->grid, b->opt};
-        if (e == cudaSuccess) e = launch_batch(b->precision, b->integrator, L, cap);
+        if (e == cudaSuccess) e = launch_batch(b->precision, b->mode, L, cap);
         cudaGraph_t g = nullptr;
         const cudaError_t e2 = cudaStreamEndCapture(cap, &g);
         cudaStreamDestroy(cap);
@@ -376,6 +405,7 @@ int rt_batch_render(rt_batch* b, float* const* d_rgb, void* stream)
         b->graph = g;
         RT_CK(cudaGraphInstantiate(&b->exec, b->graph, 0));
         b->graph_min_active = b->min_active;
+        b->graph_mode = b->mode;
     }
     RT_CK(cudaGraphLaunch(b->exec, st));
     RT_CK(cudaEventRecord(b->done, st));
@@ -449,7 +479,7 @@ int rt_batch_autotune(rt_batch* b, float* const* d_rgb, int32_t trials, void* st
     if (!tune_lookup(key, &v, &m)) {
         const int cand[] = {12, 16, 20, 24, 28};
         float best = 1e30f;
-        m = default_min_active(b->precision, b->integrator);
+        m = default_min_active(b->precision, b->mode);
         for (int c : cand) {
             b->min_active = c;
             float ms = 0.0f;

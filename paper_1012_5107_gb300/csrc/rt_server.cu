@@ -52,7 +52,8 @@ constexpr int kRingSlots = 1024;          // requests a ring holds in flight
 constexpr int kRingGrabTries = 4096;      // scans of one grab before it gives up
 constexpr int kRingWindow = 64;           // oldest requests with samples left that a grab chooses from
 constexpr int kRingLocalBits = 40;        // a grabbed sample: slot << 40 | its index in the request
-constexpr int kRingKinds = 6;             // precision x integrator (RK4, DP45, RK4T)
+constexpr int kRingKinds = 8;             // precision x integrator (RK4, DP45, RK4T), then FP64 RK4 and DP45 scenes
+                                          // within the split steps' bounds (kModeSplit)
 
 // One published request (device memory).
 struct RingSlot {
@@ -246,7 +247,7 @@ static cudaError_t ring_occupancy_t(int* bps)
                                                          WaveShape<R, INTEG>::kBlock, wave_smem_bytes<R, INTEG>());
 }
 
-static int kind_of(int precision, int integrator) { return precision * 3 + integrator; }
+static int kind_of(int precision, int mode) { return (mode & kModeSplit) ? 6 + (mode & 7) : precision * 3 + mode; }
 
 static cudaError_t ring_launch(int kind, int grid, RingSlot* slots, RingCtl* ctl, RingDone* done,
                                unsigned long long* counters, cudaStream_t st)
@@ -257,6 +258,8 @@ static cudaError_t ring_launch(int kind, int grid, RingSlot* slots, RingCtl* ctl
         case 2: return ring_launch_t<float, RT_RK4T>(grid, slots, ctl, done, counters, st);
         case 3: return ring_launch_t<double, RT_RK4>(grid, slots, ctl, done, counters, st);
         case 4: return ring_launch_t<double, RT_DP45>(grid, slots, ctl, done, counters, st);
+        case 6: return ring_launch_t<double, RT_RK4 | kModeSplit>(grid, slots, ctl, done, counters, st);
+        case 7: return ring_launch_t<double, RT_DP45 | kModeSplit>(grid, slots, ctl, done, counters, st);
         default: return ring_launch_t<double, RT_RK4T>(grid, slots, ctl, done, counters, st);
     }
 }
@@ -269,6 +272,8 @@ static cudaError_t ring_occupancy(int kind, int* bps)
         case 2: return ring_occupancy_t<float, RT_RK4T>(bps);
         case 3: return ring_occupancy_t<double, RT_RK4>(bps);
         case 4: return ring_occupancy_t<double, RT_DP45>(bps);
+        case 6: return ring_occupancy_t<double, RT_RK4 | kModeSplit>(bps);
+        case 7: return ring_occupancy_t<double, RT_DP45 | kModeSplit>(bps);
         default: return ring_occupancy_t<double, RT_RK4T>(bps);
     }
 }
@@ -630,7 +635,7 @@ static void worker_main(rt_server* S)
         if (S->stop && S->in_flight == 0 && !any_launch_running(S)) break;
         // admit in arrival order while the budget, the ring and the arena
         // allow, letting a request that fits pass ones that do not (kMaxPassed)
-        bool touched[kRingKinds] = {false, false, false, false, false, false};
+        bool touched[kRingKinds] = {};
         size_t qi = 0;
         while (!S->stop && qi < S->queue.size() && qi < kAdmitLookahead) {
             Request& r = S->req[S->queue[qi]];
@@ -815,7 +820,9 @@ int rt_submit(rt_server* S, const rt_scene_desc* desc, float* d_out, uint64_t* t
     r.bytes = request_bytes(&d);
     r.arena_off = r.arena_bytes = 0;
     r.cnt_off = r.cnt_bytes = 0;
-    r.kind = kind_of(d.precision, d.integrator);
+    DevScene table;
+    build_scene_table(&d, &table);
+    r.kind = kind_of(d.precision, wave_mode(d.precision, d.integrator, table));
     r.seq = 0;
     r.nsamples = 0;
     r.status = RT_PENDING;

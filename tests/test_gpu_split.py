@@ -106,3 +106,41 @@ def test_wide_stages_equal_general_step(over):
     assert np.abs(a["pos"] - b["pos"]).max() <= 1e-10 * p["Lambda"]
     assert np.abs(a["dir"] - b["dir"]).max() <= 1e-10
     assert np.array_equal(a_rgb, b_rgb)
+
+
+@pytest.mark.parametrize("integrator", [0, 1])
+def test_batches_and_server_take_the_same_steps(integrator):
+    """FP64 batches (all scenes within the bounds, one past them, an update from
+    one to the other and back) and served requests equal the renders alone."""
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    base = dict(precision=1, integrator=integrator, rtol=1e-7, atol=1e-7, spp=4, seed=3)
+    inside = [inputs.base_scene(width=40, height=28, **base), inputs.base_scene(width=33, height=20, A=0.02, azim_deg=20.0, **base)]
+    past = [inside[0], dict(inside[1], A=0.05)]          # kA = 0.314
+    bare = inputs.three_renders(inside[0])["bare"]
+
+    def alone(p):
+        sc = rt.Scene(p)
+        rgb = torch.zeros(sc.shape, dtype=torch.float32, device="cuda")
+        sc.render(rgb)
+        return rgb.cpu().numpy()
+
+    ref = {k: [alone(p) for p in ps] for k, ps in (("inside", inside + [bare]), ("past", past + [bare]))}
+    scenes = [rt.Scene(p) for p in inside + [bare]]
+    img = [torch.zeros(s.shape, dtype=torch.float32, device="cuda") for s in scenes]
+    b = rt.Batch(scenes)
+    for kind, ps in (("inside", inside), ("past", past), ("inside", inside)):
+        b.update(ps + [bare])
+        b.render(img)
+        for t, r in zip(img, ref[kind]):
+            assert np.array_equal(t.cpu().numpy(), r)
+    assert b.stats()["sched_timeouts"] == 0
+    s = rt.Server(1 << 28, max_inflight=2)
+    out = [torch.zeros(sc.shape, dtype=torch.float32, device="cuda") for sc in scenes[:2] for _ in range(2)]
+    tickets = [s.submit(p, t) for p, t in zip([inside[0], past[0], inside[1], past[1]], out)]
+    for t in tickets:
+        while s.poll(t, 1_000_000) is None:
+            pass
+    for t, r in zip(out, [ref["inside"][0], ref["past"][0], ref["inside"][1], ref["past"][1]]):
+        assert np.array_equal(t.cpu().numpy(), r)
+    s.close()
