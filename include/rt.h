@@ -233,7 +233,10 @@ int rt_scene_stats(rt_scene* scene, rt_stats* out);
  *               warps; the only one for RT_RK4T and for scenes with
  *               flags); -1 keeps the current one
  *   min_active  the integration loop of a warp continues while at least this
- *               many of its 32 lanes are inside the cloak (1..32); 0 keeps it
+ *               many of its 32 lanes are inside the cloak (1..32); 0 keeps it.
+ *               The wavefront loop's FP32 builds, and its FP64 builds in two
+ *               and three floats, run their loops to the end while there are
+ *               samples to start, and heed it after that
  * Returns RT_EINVAL for values out of range or a variant not compiled for the
  * scene's precision and integrator.
  */

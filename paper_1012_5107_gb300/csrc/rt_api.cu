@@ -93,6 +93,7 @@ struct rt_scene {
     int nsm;
     int variant;              // launch variant of the render (per-lane loop or wavefront loop)
     int min_active;           // lanes inside the cloak that keep the integration loop going
+    bool min_active_set;      // by the caller (a default follows the variant)
     int grid;
     float* d_tex;
     unsigned long long* d_counters;
@@ -607,8 +608,14 @@ int rt_scene_set_launch(rt_scene* s, int32_t variant, int32_t min_active)
         RT_REQ(bps > 0, "variant %d does not fit on this device", variant);
         s->variant = variant;
         s->grid = bps * s->nsm;
+        if (!s->min_active_set)
+            s->min_active = default_min_active(
+                s->desc.precision, wave_mode(s->desc.precision, render_mode(s->desc), s->dev), variant);
     }
-    if (min_active > 0) s->min_active = min_active;
+    if (min_active > 0) {
+        s->min_active = min_active;
+        s->min_active_set = true;
+    }
     return RT_OK;
 }
 

@@ -8,9 +8,10 @@
 // rays that need service (an event located, a sample finished, a new pixel).
 // Each warp repeatedly takes one task:
 //   * integrate: up to 32 rays from the cloak queue, stepped together until
-//     fewer than min_active (scaled to the rays taken) are still inside or the
-//     step cap of a task is reached; the rays still inside go back to the
-//     cloak queue, the others to the service queue;
+//     none is inside any more, or, once the work list has run dry, until fewer
+//     than min_active (scaled to the rays taken) are or a step cap is reached;
+//     the rays still inside go back to the cloak queue, the others to the
+//     service queue (see kWaveTaskSteps);
 //   * serve: up to 32 entries of the service queue, filled up with free pool
 //     entries that take new samples; each lane runs the service steps of
 //     rt_trace.cuh until its ray is inside the cloak again (back to the cloak
@@ -33,10 +34,22 @@
 
 namespace grt {
 
-// Step cap of one integration task: the rays still inside go back to the
-// cloak queue after it, and the warp takes its next task (the step's batched
-// launch, CUDA events: 7.10 ms at 128, 7.14 at 96, 7.29 at 64, 7.16 at 256,
-// 7.28 at 512, 7.34 at 1024)
+// An integration task runs to its end while the work list lasts: until none of
+// its rays is inside any more.  Its rays came from neighbouring samples and
+// stay together, so their steps take the same branches and end at about the
+// same time; a task cut short hands its stragglers on one by one, and they
+// break up the tasks after it (from 1 to 2 rays left behind the 1920 x 1080 x 16
+// render goes from 85.6 to 114.8 ms).  Once the list has run dry, what is left
+// are the longest rays, and a ray that needs service must not wait for the
+// others of its task: the rays still inside go back to the cloak queue every
+// kWaveTaskSteps steps, or when fewer than min_active (scaled to the rays taken)
+// are inside.  Measured, cut throughout at each medium's best min_active and so:
+// the step's launch 7.00 / 6.54 ms, E = 2 / 8 / 32 Dormand-Prince 18.4 / 111.6 /
+// 202.0 and 15.5 / 85.3 / 172.6, the Gaussian render 8.59 / 8.23, the time form
+// 8.65 / 8.69, 64 scenes 725 / 706, the split FP64 render 39.1 / 37.8; uncut to the
+// very end 64 x 64 x 1 takes 1.5 ms instead of 1.3.  The general FP64 builds, bound
+// by the FP64 pipe, whose instructions cost the same for few lanes as for all,
+// are cut throughout.
 constexpr int kWaveTaskSteps = 128;
 constexpr int kWaveSpin = kDefaultWaitSpin;  // attempts (with a short sleep) before a wait gives up
 
@@ -59,6 +72,7 @@ struct WaveShape {
     static constexpr bool kDp = sizeof(R) == 4 && integ_of(INTEG) == RT_DP45;
     static constexpr bool kWide = kDp && gauss_of(INTEG);
     static constexpr bool kInPool = kDp && !gauss_of(INTEG);
+    static constexpr bool kUncut = sizeof(R) == 4 || (INTEG & kModeSplit) != 0;   // see kWaveTaskSteps
     static constexpr int kBlock = kWide ? 384 : 256;
     static constexpr int kMinBlocks = ((sizeof(R) == 4 && !kWide) || split_of(INTEG)) ? 2 : 1;
     static constexpr int P = kWide ? 576 : (sizeof(R) == 4 ? 384 : (split_of(INTEG) ? 280 : 320));
@@ -200,10 +214,16 @@ __device__ __forceinline__ void wave_finish_sample(const Src& src, const DevScen
     src.pixel_done(C.scene);
 }
 
+// Whether the work list has run dry (warp-uniform).
+__device__ __forceinline__ bool wave_exhausted(const WaveCtl& Q)
+{
+    return __any_sync(0xffffffffu, *(volatile const int*)&Q.exhausted);
+}
+
 // The integration task of the split double precision step: the rays' states
 // are SplitBoxes, stepped as in the general task of wave_loop.
-__device__ __forceinline__ void wave_split_task(const DevScene& sc, Cold<double>& C, int p, SplitBox* boxes, int m1,
-                                                int min_active, int& dest, LaneStats& st,
+__device__ __forceinline__ void wave_split_task(const DevScene& sc, Cold<double>& C, int p, SplitBox* boxes, int need,
+                                                const WaveCtl& Q, bool open, int& dest, LaneStats& st,
                                                 unsigned long long* iters)
 {
     SplitBox& e = boxes[p >= 0 ? p : 0];
@@ -213,16 +233,16 @@ __device__ __forceinline__ void wave_split_task(const DevScene& sc, Cold<double>
         surf = C.surf;
         steps = C.steps;
     }
-    const int need = max(1, m1 - (32 - min_active));
     const F2 kappa = sc.sp.kappa;
     const int64_t max_steps = sc.max_steps;
     int safe = 0;
-    for (int it = 0; it < kWaveTaskSteps; ++it) {
+    for (int it = 1;; ++it) {
 #if RT_PROFILE
         ++*iters;
 #endif
         if (phase == PH_BOX) split_box_step(sc, kappa, max_steps, C, e, phase, surf, steps, st, safe);
         if (__popc(__ballot_sync(0xffffffffu, phase == PH_BOX)) < need) break;
+        if (it % kWaveTaskSteps == 0 && (!open || wave_exhausted(Q))) break;
     }
     if (p >= 0) {
         C.surf = surf;
@@ -277,6 +297,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
     for (;;) {
         // ---- take a task (the leader decides under the lock) ----
         int task = WT_WAIT, m1 = 0, m2 = 0, b1 = 0, b2 = 0, locked = 0;
+        int open = 0;                  // integrate: the work list lasts
         if (lane == 0) {
             if (!wave_acquire(&Q.lock, ww.spin)) {
                 task = WT_ERR;
@@ -297,6 +318,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
                     b2 = Q.fr_cnt;
                 } else if (nin > 0) {
                     task = WT_INT;
+                    open = WaveShape<R, INTEG>::kUncut && !Q.exhausted;
                     m1 = min(32, nin);
                     b1 = Q.in_head;
                     Q.in_head = (Q.in_head + m1) % P;
@@ -313,6 +335,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
         m2 = __shfl_sync(0xffffffffu, m2, 0);
         b1 = __shfl_sync(0xffffffffu, b1, 0);
         b2 = __shfl_sync(0xffffffffu, b2, 0);
+        if constexpr (WaveShape<R, INTEG>::kUncut) open = __shfl_sync(0xffffffffu, open, 0);
         int p = -1;
         bool fresh = false;
         if (task == WT_INT && (int)lane < m1) p = inq[(b1 + (int)lane) % P];
@@ -348,7 +371,8 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
 #if RT_PROFILE
             iters = &prof[2];
 #endif
-            if constexpr (split_of(INTEG)) wave_split_task(sc, C, p, boxes, m1, min_active, dest, st, iters);
+            if constexpr (split_of(INTEG))
+                wave_split_task(sc, C, p, boxes, open ? 1 : max(1, m1 - (32 - min_active)), Q, open != 0, dest, st, iters);
         } else if (task == WT_INT) {
             // ---- integrate ----
             if constexpr (!split_of(INTEG)) {
@@ -359,7 +383,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
                 surf = C.surf;
                 steps = C.steps;
             }
-            const int need = max(1, m1 - (32 - min_active));
+            const int need = open ? 1 : max(1, m1 - (32 - min_active));
             // step constants: read in place from the kernel parameters, or
             // copied once per task from a scene table in device memory
             const StepConst<R>* kp = &step_const<R>(sc);
@@ -370,7 +394,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
             }
             const int64_t max_steps = sc.max_steps;
             int safe = 0;                          // steps without the faces' tests (box_step_into)
-            for (int it = 0; it < kWaveTaskSteps; ++it) {
+            for (int it = 1;; ++it) {
 #if RT_PROFILE
                 prof[2] += 1;
 #endif
@@ -381,6 +405,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
                         box_step<R, INTEG>(*kp, max_steps, C, b, phase, surf, steps, st, safe);
                 }
                 if (__popc(__ballot_sync(0xffffffffu, phase == PH_BOX)) < need) break;
+                if (it % kWaveTaskSteps == 0 && (!open || wave_exhausted(Q))) break;
             }
             if (p >= 0) {
                 if constexpr (!WaveShape<R, INTEG>::kInPool) boxes[p] = b;
