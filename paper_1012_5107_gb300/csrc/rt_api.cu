@@ -42,16 +42,24 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t stream)
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
             props.location.id = dev;
-            cudaMemPool_t made;
-            e = cudaMemPoolCreate(&made, &props);
+            // The first use may fall within a stream capture, of this thread or
+            // of another, which must not end for it: making a pool enqueues
+            // nothing, so it is safe there, but a capture forbids it unless the
+            // calling thread is in relaxed mode.
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            e = cudaThreadExchangeStreamCaptureMode(&mode);
             if (e != cudaSuccess) return e;
+            cudaMemPool_t made = nullptr;
             uint64_t keep = kScratchKeep;
-            e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
-            if (e != cudaSuccess) {
-                cudaMemPoolDestroy(made);
-                return e;
+            e = cudaMemPoolCreate(&made, &props);
+            if (e == cudaSuccess) {
+                e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+                if (e != cudaSuccess) cudaMemPoolDestroy(made);
             }
+            const cudaError_t e2 = cudaThreadExchangeStreamCaptureMode(&mode);
+            if (e != cudaSuccess) return e;
             g_scratch_pool[dev] = made;
+            if (e2 != cudaSuccess) return e2;
         }
         pool = g_scratch_pool[dev];
     }

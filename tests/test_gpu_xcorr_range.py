@@ -1,6 +1,9 @@
 """rt_xcorr over the ranges its three-float sums take and past them (where a
 block sums in FP64), and its column tiles, against Eqs. 14-15 in FP64."""
 import math
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -61,3 +64,42 @@ def test_xcorr_infinities_and_nan():
     out = rt.xcorr(torch.from_numpy(f).cuda(), torch.from_numpy(g).cuda(), [10.0, 50.0], 50.0).cpu().numpy()
     assert np.isfinite(out[0]).all()
     assert np.isfinite(out[1, 0]) and not np.isfinite(out[1, 1]) and np.isnan(out[1, 2]) and not np.isfinite(out[1, 3])
+
+
+CAPTURE = """
+import sys
+import torch
+from paper_1012_5107_gb300 import rt
+torch.manual_seed(3)
+f = torch.rand(200, 180, 3, device="cuda")
+g = torch.rand(200, 180, 3, device="cuda")
+out = torch.empty((3, 4) if sys.argv[1] == "xcorr" else (13, 13, 4), dtype=torch.float64, device="cuda")
+peak = torch.empty(3, dtype=torch.float64, device="cuda")
+def call(stream):
+    if sys.argv[1] == "xcorr":
+        rt.xcorr(f, g, [10.0, 25.0, 50.0], 50.0, out=out, stream=stream)
+    else:
+        rt.xcorr_map([(f, g)], 40.0, 50.0, 6, 6, out=out, peak=peak, stream=stream)
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph, capture_error_mode=sys.argv[2]):
+    call(torch.cuda.current_stream().cuda_stream)
+out.zero_()
+graph.replay()
+graph.replay()
+torch.cuda.synchronize()
+replayed = out.clone()
+call(None)
+torch.cuda.synchronize()
+assert bool(replayed.ne(0).any()) and torch.equal(replayed, out)
+"""
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+@pytest.mark.parametrize("what", ["xcorr", "map"])
+def test_first_call_under_capture(what, mode):
+    """The process's first correlation may be one that a stream capture records."""
+    pytest.importorskip("torch")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    run = subprocess.run([sys.executable, "-c", CAPTURE, what, mode], cwd=root, capture_output=True, text=True,
+                         timeout=300)
+    assert run.returncode == 0, run.stderr[-2000:]
