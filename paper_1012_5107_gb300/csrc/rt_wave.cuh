@@ -65,8 +65,11 @@ constexpr int kWaveSpin = kDefaultWaitSpin;  // attempts (with a short sleep) be
 // 1080 x 16, E = 2 / 8 / 32: 18.4 / 113.7 / 202.0 ms against 20.2 / 115.7 /
 // 204.0 with one block of 384; with the start in registers 19.4 / 125.2 /
 // 230.6).  FP32 RK4 in the pool is slower (7.07 -> 8.57 ms the step's launch:
-// its steps are a quarter as long).  The Gaussian Dormand-Prince keeps the
-// block of 384.  FP64: one block of 256 threads; the split RK4 step two.
+// its steps are a quarter as long).  Its pool holds 320 samples a block: two
+// blocks then fit the 196 KB split of the SM's memory, which leaves 60 KB of L1
+// to the spills; with 384 they need the 228 KB one and the spills miss 28 KB
+// (E = 8: 85.2 -> 80.8 ms, the same from 256 to 336 samples).  The Gaussian
+// Dormand-Prince keeps the block of 384.  FP64: one block of 256 threads; the split RK4 step two.
 template <class R, int INTEG>
 struct WaveShape {
     static constexpr bool kDp = sizeof(R) == 4 && integ_of(INTEG) == RT_DP45;
@@ -75,7 +78,7 @@ struct WaveShape {
     static constexpr bool kUncut = sizeof(R) == 4 || (INTEG & kModeSplit) != 0;   // see kWaveTaskSteps
     static constexpr int kBlock = kWide ? 384 : 256;
     static constexpr int kMinBlocks = ((sizeof(R) == 4 && !kWide) || split_of(INTEG)) ? 2 : 1;
-    static constexpr int P = kWide ? 576 : (sizeof(R) == 4 ? 384 : (split_of(INTEG) ? 280 : 320));
+    static constexpr int P = kWide ? 576 : kInPool ? 320 : (sizeof(R) == 4 ? 384 : (split_of(INTEG) ? 280 : 320));
 };
 
 static_assert((sizeof(Cold<double>) + sizeof(SplitBox) + 6) * 280 <= 115712, "two blocks of the split loop per SM");
