@@ -47,9 +47,9 @@ namespace grt {
 // the step's launch 7.00 / 6.54 ms, E = 2 / 8 / 32 Dormand-Prince 18.4 / 111.6 /
 // 202.0 and 15.5 / 85.3 / 172.6, the Gaussian render 8.59 / 8.23, the time form
 // 8.65 / 8.69, 64 scenes 725 / 706, the split FP64 render 39.1 / 37.8; uncut to the
-// very end 64 x 64 x 1 takes 1.5 ms instead of 1.3.  The general FP64 builds, bound
-// by the FP64 pipe, whose instructions cost the same for few lanes as for all,
-// are cut throughout.
+// very end 64 x 64 x 1 takes 1.52 ms instead of 1.22 (FP32 with pools of 384).
+// The general FP64 builds, bound by the FP64 pipe, whose instructions cost the
+// same for few lanes as for all, are cut throughout.
 constexpr int kWaveTaskSteps = 128;
 constexpr int kWaveSpin = kDefaultWaitSpin;  // attempts (with a short sleep) before a wait gives up
 
