@@ -7,12 +7,14 @@
 
 namespace grt {
 
-// Values that the three-float sums take: zero, or a magnitude in [2^-40, 2^60),
-// whose products neither overflow nor lose their remainders to underflow.
+// Values that the three-float sums take: zero, or a magnitude in [2^-40, 2^48).
+// The products' remainders stay clear of underflow, and the products, below
+// 2^96, of overflow in any sum of up to 2^31 of them: a column's sum runs over
+// the rows of a chunk, which may be the whole image.
 __device__ __forceinline__ bool xcorr_plain(float v)
 {
     const uint32_t u = __float_as_uint(v) & 0x7fffffffu;
-    return u == 0u || u - (87u << 23) < (100u << 23);
+    return u == 0u || u - (87u << 23) < (88u << 23);
 }
 
 // Three-float running sums of a pair of values; xcorr_low adds remainders.

@@ -103,3 +103,25 @@ def test_first_call_under_capture(what, mode):
     run = subprocess.run([sys.executable, "-c", CAPTURE, what, mode], cwd=root, capture_output=True, text=True,
                          timeout=300)
     assert run.returncode == 0, run.stderr[-2000:]
+
+
+# The largest values whose products FP32 holds, over chunks of more rows than
+# FP32 holds sums of (2^128 / 2^120 = 256), and the edge of the three-float
+# range.  The tolerance is test_xcorr_ranges'.
+@pytest.mark.parametrize("H,W,C,scale", [
+    (1200, 9729, 1, 2.0 ** 59.9),                        # one chunk of all rows (W C >= 9728)
+    (2160, 3840, 3, 2.0 ** 59.9), (1080, 1920, 3, 2.0 ** 48), (700, 9728, 1, 2.0 ** 47.9),
+    (4096, 70, 1, 2.0 ** 59.9),
+])
+def test_xcorr_tall_chunks_of_large_values(H, W, C, scale):
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    rng = np.random.default_rng([H, W, C, 1])
+    f = (0.5 + 0.5 * rng.random((H, W, C))).astype(np.float32)
+    g = (0.7 * f + 0.3 * rng.random((H, W, C))).astype(np.float32)
+    f, g = (f * np.float32(scale)).astype(np.float32), (g * np.float32(scale)).astype(np.float32)
+    tf, tg = torch.from_numpy(f).cuda(), torch.from_numpy(g).cuda()
+    ref = [c00(f, g, columns(W, 50.0, fov)) for fov in (25.0, 50.0)]
+    for call in (rt.xcorr, rt.xcorr_noalloc):
+        out = call(tf, tg, [25.0, 50.0], 50.0).cpu().numpy()
+        assert np.abs(out - np.array(ref)).max() < 1e-11
