@@ -405,7 +405,8 @@ int rt_server_stats(rt_server* server, rt_server_info* out);
  * channel c: C_c = sum (f-<f>)(g-<g>) / sum (f-<f>)^2 with the means over the
  * window (Eq. 14); the last entry treats the channels as one stacked image.
  * Writes n_fov x (channels+1) doubles to d_out (device).  Empty windows give
- * NaN.  Asynchronous; uses scratch owned by the library.
+ * NaN.  width * channels is at most 2^31 - 32.  Asynchronous; uses scratch
+ * owned by the library.
  */
 int rt_xcorr(const float* d_f, const float* d_g, int32_t height, int32_t width, int32_t channels,
              const double* fov_deg, int32_t n_fov, double hfov_deg, double* d_out, void* stream);

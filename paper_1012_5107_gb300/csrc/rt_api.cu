@@ -655,6 +655,7 @@ int rt_xcorr(const float* d_f, const float* d_g, int32_t height, int32_t width, 
     RT_REQ(d_f && d_g && d_out && fov_deg, "null pointer argument");
     RT_REQ(height >= 1 && width >= 1, "height and width must be >= 1");
     RT_REQ(channels >= 1 && channels <= 4, "channels must be 1..4");
+    RT_REQ((int64_t)width * channels <= kXcorrMaxRow, "width * channels must be <= %lld", (long long)kXcorrMaxRow);
     RT_REQ(n_fov >= 1 && n_fov <= kMaxWindows, "n_fov must be 1..%d", kMaxWindows);
     RT_REQ(hfov_deg > 0.0 && hfov_deg < 180.0, "hfov_deg must be in (0, 180)");
     for (int q = 0; q < n_fov; ++q) RT_REQ(fov_deg[q] >= 0.0, "fov_deg must be >= 0");

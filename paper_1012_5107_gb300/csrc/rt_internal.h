@@ -116,6 +116,8 @@ cudaError_t launch_medium(int precision, double kA, double Lambda, const double*
 // xcorr_scratch_bytes(...) bytes, at most kXcorrScratch (none for the small
 // images that one block takes).
 constexpr size_t kXcorrScratch = (size_t)5 << 18;
+// Values of a row: the kernels index them, and the 32-column tiles behind them, in 32 bits.
+constexpr int64_t kXcorrMaxRow = (int64_t)0x7fffffff - 31;
 size_t xcorr_scratch_bytes(int H, int W, int C, int n_fov);
 // Scratch of the correlation calls, in stream order, from a pool of the
 // library's own that keeps up to kScratchKeep bytes between calls (the default

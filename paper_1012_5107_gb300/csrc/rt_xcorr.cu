@@ -44,7 +44,7 @@ static_assert(kXcorrScratch >= (size_t)2 * kXcorrBlocks * kMaxWindows * 16 * siz
 static dim3 xcorr_grid(int H, int W, int C)
 {
     const int64_t tiles = std::min<int64_t>(((int64_t)W * C + 31) / 32, kXcorrBlocks);
-    const int64_t chunks = std::min<int64_t>((kXcorrBlocks + tiles - 1) / tiles, (H + kXcorrWarps - 1) / kXcorrWarps);
+    const int64_t chunks = std::min<int64_t>((kXcorrBlocks + tiles - 1) / tiles, ((int64_t)H + kXcorrWarps - 1) / kXcorrWarps);
     return dim3((unsigned)tiles, (unsigned)chunks);
 }
 
@@ -142,7 +142,10 @@ __global__ void __launch_bounds__(kXcorrBlock) xcorr_moments(const float* __rest
     const bool mine = w < win.n;
     const int j0 = mine ? win.j0[w] : 0, j1 = mine ? win.j1[w] : 0;
     double acc = 0.0;
-    for (int q0 = blockIdx.x * 32; q0 < WC; q0 += gridDim.x * 32) {
+    // (counted in tiles: q0 would pass 2^31 behind a row that nearly fills it)
+    const int tiles = (int)(((int64_t)WC + 31) / 32);
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int q0 = tile * 32;
         xcorr_tile(f, g, WC, q0, i0, i1, red3, col);
         __syncthreads();
         // the tile's columns of channel c: pixels (q0 + l) / C, l = first, first + C, ...
@@ -270,7 +273,7 @@ cudaError_t launch_xcorr(const float* f, const float* g, int H, int W, int C, co
         return cudaGetLastError();
     }
     const dim3 grid = xcorr_grid(H, W, C);
-    const int rpc = (H + (int)grid.y - 1) / (int)grid.y;
+    const int rpc = (int)(((int64_t)H + grid.y - 1) / grid.y);
     xcorr_moments<<<grid, kXcorrBlock, 0, stream>>>(f, g, H, W, C, rpc, win, (double*)scratch);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -301,7 +304,7 @@ void fov_windows(int W, double hfov_deg, const double* fov_deg, int n_fov, Windo
         }
         int c = mid - 1, d = W - 1;           // the last column inside in [mid - 1, W - 1], or mid - 1
         while (c < d) {
-            const int m = (c + d + 1) / 2;
+            const int m = c + (d - c + 1) / 2;                // (c + d may pass 2^31)
             if (inside(m)) c = m;
             else d = m - 1;
         }

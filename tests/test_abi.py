@@ -108,3 +108,22 @@ def test_request_bytes_rejects_invalid(rt):
     with pytest.raises(rt.RtError) as e:
         rt.request_bytes(inputs.base_scene(width=0))
     assert e.value.code == rt.RT_EINVAL
+
+
+def test_rows_past_the_index_range_are_refused(rt):
+    """Rows of more values than 32-bit indices reach are refused before any launch."""
+    import ctypes as C
+    fov, p = (C.c_double * 1)(50.0), C.c_void_p(256)            # (no pointer is followed)
+    for width, channels in ((2 ** 31 - 1, 1), (2 ** 31 - 31, 1), (2 ** 30, 4), (2 ** 30, 2), (2 ** 31 - 1, 3)):
+        rc = rt.lib().rt_xcorr(p, p, 1, width, channels, fov, 1, 50.0, p, None)
+        assert rc == rt.RT_EINVAL and b"width * channels" in rt.lib().rt_last_error()
+
+
+def test_columns_of_the_widest_image(rt):
+    """The bisection for the window's columns at widths whose sums of two column
+    indices pass 2^31: the centre column alone at a field of view of 0 (the call
+    is refused for its height, after the columns were found)."""
+    import ctypes as C
+    ptrs = (C.c_void_p * 1)(256)
+    rc = rt.lib().rt_xcorr_map(ptrs, ptrs, 1, 8 * 65536, 2 ** 31 - 1, 1, 0.0, 50.0, 0, 0, C.c_void_p(256), None, None)
+    assert rc == rt.RT_EINVAL and b"65536 x 1 window chunks" in rt.lib().rt_last_error()
