@@ -25,6 +25,7 @@
 // FP32 peak).  +-31 x +-3 shifts of two 326 x 164 pairs 139 -> 58 us, +-40 of two
 // 300 x 400 x 3 pairs 1,095 -> 312 us.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <vector>
 
@@ -37,6 +38,11 @@ constexpr int kMapRows = 8;       // image rows per chunk
 constexpr int kMapCols = 128;     // image columns per chunk
 constexpr int kMapThreads = 160;  // threads per block of the tiles, at most
 constexpr int kMapMaxShift = 64;
+// Shared memory of any plan (the largest over all shifts and heights: 107,284
+// bytes).  The limit of a kernel is the process's, so it is set to this once and
+// not to a call's own size: a smaller call of another thread would lower it
+// between a larger call's setting and its launch.
+constexpr size_t kMapSmem = 108 * 1024;
 
 // How a launch of the tiles is laid out: a thread owns RI x RJ shifts, gi x gj
 // threads the shifts of a chunk, of which a block takes git along di; kc row
@@ -405,8 +411,17 @@ static cudaError_t launch_tiles(cudaStream_t st, const MapPlan& p, const MapImag
                                float* part)
 {
     if (p.ri != RI || p.rj != RJ) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(xmap_tiles<RI, RJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    if (p.smem > kMapSmem) return cudaErrorInvalidValue;
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(done.load() & bit)) {
+        e = cudaFuncSetAttribute(xmap_tiles<RI, RJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMapSmem);
+        if (e != cudaSuccess) return e;
+        done.fetch_or(bit);
+    }
     const dim3 grid((unsigned)(((p.gi + p.git - 1) / p.git) * ((nrc + p.kc - 1) / p.kc) * ncc), npc);
     xmap_tiles<RI, RJ><<<grid, p.threads, p.smem, st>>>(im, stats, H, W, C, j0, j1, max_di, max_dj, nrc, ncc, p, part);
     return cudaGetLastError();

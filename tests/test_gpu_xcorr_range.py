@@ -125,3 +125,39 @@ def test_xcorr_tall_chunks_of_large_values(H, W, C, scale):
     for call in (rt.xcorr, rt.xcorr_noalloc):
         out = call(tf, tg, [25.0, 50.0], 50.0).cpu().numpy()
         assert np.abs(out - np.array(ref)).max() < 1e-11
+
+
+def test_maps_of_two_threads_at_once():
+    """Calls whose tiles need different amounts of shared memory, alternated on two
+    threads' streams, give what they give alone."""
+    torch = pytest.importorskip("torch")
+    import threading
+
+    from paper_1012_5107_gb300 import rt
+    torch.manual_seed(5)
+    sizes = [(96, 96, 3, 40, 40), (64, 48, 1, 1, 4), (200, 300, 3, 12, 40), (40, 33, 1, 40, 13)]
+    pairs = [(torch.rand(H, W, C, device="cuda"), torch.rand(H, W, C, device="cuda")) for H, W, C, _, _ in sizes]
+    alone = [rt.xcorr_map([p], 50.0, 50.0, di, dj)[0].cpu() for p, (_, _, _, di, dj) in zip(pairs, sizes)]
+    errors = []
+
+    def work(order):
+        try:
+            stream = torch.cuda.Stream()
+            outs = [torch.empty_like(a, device="cuda") for a in alone]
+            peak = torch.empty(3, dtype=torch.float64, device="cuda")
+            torch.cuda.synchronize()
+            for _ in range(150):
+                for q in order:
+                    rt.xcorr_map([pairs[q]], 50.0, 50.0, sizes[q][3], sizes[q][4], out=outs[q], peak=peak, stream=stream)
+            stream.synchronize()
+            for a, o in zip(alone, outs):
+                assert torch.equal(a, o.cpu())
+        except Exception as e:                           # noqa: BLE001 (reported by the test's own thread)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(o,)) for o in ((0, 1, 2, 3), (3, 1, 0, 2), (2, 3, 1, 0))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
