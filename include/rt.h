@@ -234,9 +234,9 @@ int rt_scene_stats(rt_scene* scene, rt_stats* out);
  *               flags); -1 keeps the current one
  *   min_active  the integration loop of a warp continues while at least this
  *               many of its 32 lanes are inside the cloak (1..32); 0 keeps it.
- *               The wavefront loop's FP32 builds, and its FP64 builds in two
- *               and three floats, run their loops to the end while there are
- *               samples to start, and heed it after that
+ *               The wavefront loop's FP32 builds heed it where they find that
+ *               rays leave far apart, its FP64 builds in two and three floats
+ *               not at all: they run their loops to the end
  * Returns RT_EINVAL for values out of range or a variant not compiled for the
  * scene's precision and integrator.
  */

@@ -101,7 +101,6 @@ struct rt_scene {
     int nsm;
     int variant;              // launch variant of the render (per-lane loop or wavefront loop)
     int min_active;           // lanes inside the cloak that keep the integration loop going
-    bool min_active_set;      // by the caller (a default follows the variant)
     int grid;
     float* d_tex;
     unsigned long long* d_counters;
@@ -360,7 +359,7 @@ void counters_to_stats(const unsigned long long* c, rt_stats* out)
     out->fp64_refine = c[6];
     for (int q = 0; q < 5; ++q) out->status[q] = c[7 + q];
     for (int q = 0; q < 4; ++q) out->profile[q] = c[12 + q];
-    out->sched_timeouts = c[16];
+    out->sched_timeouts = c[kTimeouts];
 }
 
 }  // namespace grt
@@ -616,14 +615,8 @@ int rt_scene_set_launch(rt_scene* s, int32_t variant, int32_t min_active)
         RT_REQ(bps > 0, "variant %d does not fit on this device", variant);
         s->variant = variant;
         s->grid = bps * s->nsm;
-        if (!s->min_active_set)
-            s->min_active = default_min_active(
-                s->desc.precision, wave_mode(s->desc.precision, render_mode(s->desc), s->dev), variant);
     }
-    if (min_active > 0) {
-        s->min_active = min_active;
-        s->min_active_set = true;
-    }
+    if (min_active > 0) s->min_active = min_active;
     return RT_OK;
 }
 

@@ -17,35 +17,38 @@ constexpr int kLaneVariants = 3;
 constexpr int kVariantBlocks[kLaneVariants] = {4, 5, 6};
 constexpr int kVariantWave = 3;
 constexpr int kDefaultVariant = kVariantWave;
-// An integration task continues while at least this many of its 32 rays are
-// inside the cloak -- in the builds that run their tasks to the end while the
-// work list lasts (kWaveTaskSteps in rt_wave.cuh), only once it has run dry.
-// Measured on the current kernels (CUDA events), 1 / 8 / 24:
-//   FP32, the tail: Fresnel renders of Table 1, 256 x 256 x 4, 7.10 / 7.15 /
-//   7.96 ms; 64 x 64 x 1 RK4 1.34 / 1.33 / 1.37, Dormand-Prince 0.41 / 0.53 /
-//   0.54, Gaussian 1.97 / 2.01 / 2.11; the large renders are within 1 %;
-//   FP64 in rt_split.cuh's steps, the tail: 64 x 64 x 1 5.87 / 6.04 / 5.58,
-//   1920 x 1080 x 16 pixel subset 5.45 / 5.42 / 5.19;
-//   the general FP64 loops, bound by the FP64 pipe, with full warps only
-//   (FP64 cloaked render 590 ms at 32, 595 at 30, 605 at 28, 623 at 24), and
-//   Dormand-Prince at 8.
-// The per-lane loop (variants 0..2) refills its warps at the old values.
-constexpr int kMinActiveF32 = 1;
-constexpr int kMinActiveSplit = 24;
+// An integration task that is cut short (kWaveTaskSteps in rt_wave.cuh: the
+// general FP64 loops' always, the FP32 loops' where their rays leave far apart),
+// and the per-lane loop's, continues while at least this many of its 32 rays are
+// inside the cloak.  Measured with every task cut (CUDA events): the FP32
+// RK4 grating loop is fastest at 24 (the step's batched launch 7.25 ms, 7.34
+// at 28, 7.87 at 30); the FP32 time form and Gaussian medium at 28 (time form
+// 9.21 ms, 9.35 at 24, 9.47 at 30; Gaussian 9.39 / 9.49 ms at 28 / 24); the
+// FP64 loops, bound by the FP64 pipe, with full warps only (FP64 cloaked
+// render 590 ms at 32, 595 at 30, 605 at 28, 623 at 24).
+constexpr int kMinActive = 28;
+constexpr int kMinActiveRK4F32 = 24;
 constexpr int kMinActiveF64 = 32;
+// Dormand-Prince steps are longer: a task holding fewer rays is still worth
+// running (1920 x 1080 x 16 with one block of 384 threads per SM, E = 8 / 32:
+// 133.0 / 214.8 ms at 8, 135.1 / 221.5 ms at 16; 2 to 10 within 1 %)
 constexpr int kMinActiveDP45 = 8;
-constexpr int kMinActiveLane = 24;
-// The default for a precision (RT_FP32 / RT_FP64), render mode (the
-// integrator, with kModeGauss for the Gaussian bump, kModeSplit for the split
-// steps) and launch variant.
-inline int default_min_active(int precision, int mode, int variant = kVariantWave)
+// The default for a precision (RT_FP32 / RT_FP64) and render mode (the
+// integrator, with kModeGauss for the Gaussian bump).
+inline int default_min_active(int precision, int mode)
 {
-    if (variant != kVariantWave)
-        return (mode & 7) == RT_DP45 ? kMinActiveDP45 : precision == RT_FP64 ? kMinActiveF64 : kMinActiveLane;
-    if (precision == RT_FP32) return kMinActiveF32;
-    if (mode & 16) return kMinActiveSplit;
-    return (mode & 7) == RT_DP45 ? kMinActiveDP45 : kMinActiveF64;
+    if ((mode & 7) == RT_DP45) return kMinActiveDP45;
+    if (precision == RT_FP64) return kMinActiveF64;
+    if ((mode & 15) == RT_RK4) return kMinActiveRK4F32;
+    return kMinActive;
 }
+// Once the work list has run dry, an FP32 loop's task runs until none of its
+// rays is inside (1 / 8 / 24: Fresnel renders of Table 1, 256 x 256 x 4, 7.10 /
+// 7.15 / 7.96 ms; 64 x 64 x 1 RK4 1.34 / 1.33 / 1.37, Dormand-Prince 0.41 / 0.53 /
+// 0.54, Gaussian 1.97 / 2.01 / 2.11; the large renders are within 1 %), and one of
+// the FP64 loops in rt_split.cuh's steps while this many are (1 / 8 / 24: 64 x 64 x 1
+// 5.87 / 6.04 / 5.58 ms, 1920 x 1080 x 16 pixel subset 5.45 / 5.42 / 5.19).
+constexpr int kMinActiveSplit = 24;
 constexpr int kMaxWindows = 16;
 // Render mode: the integrator (RT_RK4, RT_DP45, RT_RK4T), with kModeGauss set
 // for scenes of the Gaussian bump, whose box holds the Gaussian map's medium.
@@ -65,8 +68,11 @@ inline int wave_mode(int precision, int mode, const DevScene& sc)
 // Coefficients of the Faddeeva series of the Gaussian cloak, uploaded once
 // per device before its first Gaussian scene.
 cudaError_t gauss_upload();
-constexpr int kCounters = 17;      // [0] work counter, [1..11] statistics, [12..15] optional profile,
-                                   // [16] wavefront-loop waits that timed out
+// [0] work counter, [1..11] statistics, [12..15] optional profile, then
+// wavefront-loop waits that timed out and the tally of wave_ragged
+constexpr int kTimeouts = 16;
+constexpr int kTally = 17;
+constexpr int kCounters = 18;
 
 #ifndef RT_PROFILE
 #define RT_PROFILE 0

@@ -584,7 +584,7 @@ static void ring_progress(rt_server* S, Ring& g)
         g.krunning[i] = false;
         unsigned long long timeouts = 0;
         if (q != cudaSuccess ||
-            cudaMemcpy(&timeouts, g.d_stats + (size_t)kCounters * i + (kCounters - 1), sizeof timeouts,
+            cudaMemcpy(&timeouts, g.d_stats + (size_t)kCounters * i + kTimeouts, sizeof timeouts,
                        cudaMemcpyDeviceToHost) != cudaSuccess)
             g.timed_out = true;
         else if (timeouts)

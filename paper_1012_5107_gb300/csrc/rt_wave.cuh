@@ -8,8 +8,8 @@
 // rays that need service (an event located, a sample finished, a new pixel).
 // Each warp repeatedly takes one task:
 //   * integrate: up to 32 rays from the cloak queue, stepped together until
-//     none is inside any more, or, once the work list has run dry, until fewer
-//     than min_active (scaled to the rays taken) are or a step cap is reached;
+//     none is inside any more, or, in a task that is cut, until fewer than
+//     min_active (scaled to the rays taken) are or a step cap is reached;
 //     the rays still inside go back to the cloak queue, the others to the
 //     service queue (see kWaveTaskSteps);
 //   * serve: up to 32 entries of the service queue, filled up with free pool
@@ -27,7 +27,7 @@
 // The queues are rings of 16-bit pool indices guarded by a block-level lock
 // (an atomic flag in shared memory) that one lane per warp takes for a few
 // dozen cycles per task; every wait on it is bounded (WaveWait) and a timeout
-// is counted in counters[kCounters - 1] (reported as an error by the host).
+// is counted in counters[kTimeouts] (reported as an error by the host).
 #pragma once
 
 #include "rt_trace.cuh"
@@ -39,15 +39,31 @@ namespace grt {
 // stay together, so their steps take the same branches and end at about the
 // same time; a task cut short hands its stragglers on one by one, and they
 // break up the tasks after it (from 1 to 2 rays left behind the 1920 x 1080 x 16
-// render goes from 85.6 to 114.8 ms).  Once the list has run dry, what is left
+// render goes from 85.6 to 114.8 ms; a queue of their own for the stragglers
+// does not help: their tasks break up one another, and the step took 7.0 ms
+// instead of 6.6).  Once the list has run dry, what is left
 // are the longest rays, and a ray that needs service must not wait for the
 // others of its task: the rays still inside go back to the cloak queue every
-// kWaveTaskSteps steps, or when fewer than min_active (scaled to the rays taken)
-// are inside.  Measured, cut throughout at each medium's best min_active and so:
-// the step's launch 7.00 / 6.54 ms, E = 2 / 8 / 32 Dormand-Prince 18.4 / 111.6 /
-// 202.0 and 15.5 / 85.3 / 172.6, the Gaussian render 8.59 / 8.23, the time form
-// 8.65 / 8.69, 64 scenes 725 / 706, the split FP64 render 39.1 / 37.8; uncut to the
-// very end 64 x 64 x 1 takes 1.52 ms instead of 1.22 (FP32 with pools of 384).
+// kWaveTaskSteps steps, or when fewer than need are inside.
+//
+// Where neighbouring rays leave far apart -- a camera that looks across the
+// grooves or at grazing elevation -- a task that waits for its last ray idles its
+// lanes: at 900 x 900 x 4, E = 32, azimuth 90 and elevation 10 degrees 49.1 ms
+// against 30.3 with tasks cut at min_active and every kWaveTaskSteps steps.  The
+// FP32 loops measure it (wave_ragged) and cut their tasks from then on: 30.4 ms.
+// Below 85 % of the lanes inside an uncut RK4 render is the slower one, above
+// 89 % the faster (Dormand-Prince, with a third of the steps between services:
+// 75 and 80 %).  The options build keeps its tasks uncut (Fresnel renders at
+// kA = 0.6 are faster so at 63 %).
+//
+// Measured, cut throughout and so: the step's launch 7.05 / 6.41 ms, E = 8 / 32
+// Dormand-Prince at 1920 x 1080 x 16 115.5 / 79.5 and 206.2 / 159.9, the Gaussian
+// render 5.63 / 5.06 (384 x 384 x 4), the time form 8.70 / 8.49, Fresnel renders
+// 7.90 / 6.02, the split FP64 render 39.1 / 37.8; uncut to the very end 64 x 64 x 1
+// takes 1.52 ms instead of 1.25.  Over 128 scenes (elevations 10 to 55, azimuths
+// 0 to 90 degrees, E = 8 and 32, kA = 0.1 and 0.25, RK4 and Dormand-Prince) it is
+// within 4 % of the better of the two at 900 x 900 x 4, and within 16 % at
+// 320 x 320 x 4, where half of the render is over before the tally tells.
 // The general FP64 builds, bound by the FP64 pipe, whose instructions cost the
 // same for few lanes as for all, are cut throughout.
 constexpr int kWaveTaskSteps = 128;
@@ -76,6 +92,7 @@ struct WaveShape {
     static constexpr bool kWide = kDp && gauss_of(INTEG);
     static constexpr bool kInPool = kDp && !gauss_of(INTEG);
     static constexpr bool kUncut = sizeof(R) == 4 || (INTEG & kModeSplit) != 0;   // see kWaveTaskSteps
+    static constexpr int kEven = integ_of(INTEG) == RT_DP45 ? 72 : 82;            // see wave_ragged
     static constexpr int kBlock = kWide ? 384 : 256;
     static constexpr int kMinBlocks = ((sizeof(R) == 4 && !kWide) || split_of(INTEG)) ? 2 : 1;
     static constexpr int P = kWide ? 576 : kInPool ? 320 : (sizeof(R) == 4 ? 384 : (split_of(INTEG) ? 280 : 320));
@@ -103,10 +120,15 @@ struct WaveCtl {
     int sv_head, sv_cnt;     // service queue
     int fr_cnt;              // free list (stack)
     int exhausted;           // the work list has no pixels left
+    int ragged;              // rays of a task leave too far apart: tasks are cut (kWaveTaskSteps)
     int error;
 };
 
 enum : int { WT_WAIT = 0, WT_INT = 1, WT_SRV = 2, WT_DONE = 3, WT_ERR = 4 };
+// Where an integration task ends: WI_OPEN when none of its rays is inside,
+// WI_CUT when fewer than min_active are or after kWaveTaskSteps, WI_LAST (the
+// list has run dry) as the build does best.
+enum : int { WI_LAST = 0, WI_CUT = 1, WI_OPEN = 2 };
 enum : int { WD_NONE = 0, WD_IN = 1, WD_SRV = 2, WD_FREE = 3 };
 
 // How the waits of a launch are bounded: `spin` attempts per wait (kWaveSpin
@@ -223,6 +245,28 @@ __device__ __forceinline__ bool wave_exhausted(const WaveCtl& Q)
     return __any_sync(0xffffffffu, *(volatile const int*)&Q.exhausted);
 }
 
+// Counts `its` steps of an uncut FP32 task of 32 rays, `lanes` of them by lanes
+// still inside, and says whether such tasks kept fewer than kEven percent of
+// their lanes inside of late, over all blocks of the launch.  The tally (steps,
+// and lanes / 32, in halves of a word) is halved when it reaches kTallySteps,
+// about a task's length of every warp, so it follows the work; a launch's first
+// tasks, whose early steps have all lanes inside, do not weigh on it for long.
+constexpr unsigned kTallySteps = 1u << 19;
+__device__ __forceinline__ bool wave_ragged(unsigned long long* counters, unsigned its, unsigned lanes, int even)
+{
+    unsigned long long now = 0;
+    if ((threadIdx.x & 31u) == 0) {
+        const unsigned long long add = ((unsigned long long)its << 32) + ((lanes + 16u) >> 5);
+        const unsigned long long old = atomicAdd(&counters[kTally], add);
+        now = old + add;
+        if ((unsigned)(old >> 32) < kTallySteps && (unsigned)(now >> 32) >= kTallySteps)
+            atomicAdd(&counters[kTally], 0ull - (((now >> 33) << 32) + ((now & 0xffffffffull) >> 1)));
+    }
+    now = __shfl_sync(0xffffffffu, now, 0);
+    const unsigned long long n = now >> 32;
+    return n > kTallySteps / 4 && (now & 0xffffffffull) * 100ull < n * (unsigned)even;
+}
+
 // The integration task of the split double precision step: the rays' states
 // are SplitBoxes, stepped as in the general task of wave_loop.
 __device__ __forceinline__ void wave_split_task(const DevScene& sc, Cold<double>& C, int p, SplitBox* boxes, int need,
@@ -283,6 +327,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
         Q.in_head = Q.in_cnt = Q.sv_head = Q.sv_cnt = 0;
         Q.fr_cnt = P;
         Q.exhausted = 0;
+        Q.ragged = 0;
         Q.error = 0;
     }
     __syncthreads();
@@ -300,7 +345,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
     for (;;) {
         // ---- take a task (the leader decides under the lock) ----
         int task = WT_WAIT, m1 = 0, m2 = 0, b1 = 0, b2 = 0, locked = 0;
-        int open = 0;                  // integrate: the work list lasts
+        int how = WI_LAST;             // integrate: where the task ends
         if (lane == 0) {
             if (!wave_acquire(&Q.lock, ww.spin)) {
                 task = WT_ERR;
@@ -321,7 +366,8 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
                     b2 = Q.fr_cnt;
                 } else if (nin > 0) {
                     task = WT_INT;
-                    open = WaveShape<R, INTEG>::kUncut && !Q.exhausted;
+                    if constexpr (WaveShape<R, INTEG>::kUncut)
+                        how = Q.exhausted ? WI_LAST : Q.ragged ? WI_CUT : WI_OPEN;
                     m1 = min(32, nin);
                     b1 = Q.in_head;
                     Q.in_head = (Q.in_head + m1) % P;
@@ -338,7 +384,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
         m2 = __shfl_sync(0xffffffffu, m2, 0);
         b1 = __shfl_sync(0xffffffffu, b1, 0);
         b2 = __shfl_sync(0xffffffffu, b2, 0);
-        if constexpr (WaveShape<R, INTEG>::kUncut) open = __shfl_sync(0xffffffffu, open, 0);
+        if constexpr (WaveShape<R, INTEG>::kUncut) how = __shfl_sync(0xffffffffu, how, 0);
         int p = -1;
         bool fresh = false;
         if (task == WT_INT && (int)lane < m1) p = inq[(b1 + (int)lane) % P];
@@ -375,7 +421,8 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
             iters = &prof[2];
 #endif
             if constexpr (split_of(INTEG))
-                wave_split_task(sc, C, p, boxes, open ? 1 : max(1, m1 - (32 - min_active)), Q, open != 0, dest, st, iters);
+                wave_split_task(sc, C, p, boxes, how == WI_OPEN ? 1 : max(1, m1 - (32 - kMinActiveSplit)), Q, how == WI_OPEN,
+                                dest, st, iters);
         } else if (task == WT_INT) {
             // ---- integrate ----
             if constexpr (!split_of(INTEG)) {
@@ -386,7 +433,9 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
                 surf = C.surf;
                 steps = C.steps;
             }
-            const int need = open ? 1 : max(1, m1 - (32 - min_active));
+            int need = 1;
+            if (!WaveShape<R, INTEG>::kUncut || how == WI_CUT) need = max(1, m1 - (32 - min_active));
+            else if (sizeof(R) == 8 && how == WI_LAST) need = max(1, m1 - (32 - kMinActiveSplit));
             // step constants: read in place from the kernel parameters, or
             // copied once per task from a scene table in device memory
             const StepConst<R>* kp = &step_const<R>(sc);
@@ -397,18 +446,35 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
             }
             const int64_t max_steps = sc.max_steps;
             int safe = 0;                          // steps without the faces' tests (box_step_into)
-            for (int it = 1;; ++it) {
+            // stretches of kWaveTaskSteps steps (the loop within has no more
+            // tests than a cut task needs: with the stretch's end tested in it
+            // the step took 2 to 3 % longer)
+            for (;;) {
+                const int before = steps;
+                int it = 0, inside = 0;
+                for (; it < kWaveTaskSteps; ++it) {
 #if RT_PROFILE
-                prof[2] += 1;
+                    prof[2] += 1;
 #endif
-                if (phase == PH_BOX) {
-                    if constexpr (WaveShape<R, INTEG>::kInPool)
-                        box_step<R, INTEG>(*kp, max_steps, C, boxes[p], phase, surf, steps, st, safe);
-                    else
-                        box_step<R, INTEG>(*kp, max_steps, C, b, phase, surf, steps, st, safe);
+                    if (phase == PH_BOX) {
+                        if constexpr (WaveShape<R, INTEG>::kInPool)
+                            box_step<R, INTEG>(*kp, max_steps, C, boxes[p], phase, surf, steps, st, safe);
+                        else
+                            box_step<R, INTEG>(*kp, max_steps, C, b, phase, surf, steps, st, safe);
+                    }
+                    inside = __popc(__ballot_sync(0xffffffffu, phase == PH_BOX));
+                    if (inside < need) { ++it; break; }
                 }
-                if (__popc(__ballot_sync(0xffffffffu, phase == PH_BOX)) < need) break;
-                if (it % kWaveTaskSteps == 0 && (!open || wave_exhausted(Q))) break;
+                if (!WaveShape<R, INTEG>::kUncut || how != WI_OPEN) break;
+                bool ragged = false;
+                if constexpr (sizeof(R) == 4 && !OPT) {
+                    if (m1 == 32) {
+                        const unsigned lanes = __reduce_add_sync(0xffffffffu, (unsigned)(steps - before));
+                        ragged = wave_ragged(counters, (unsigned)it, lanes, WaveShape<R, INTEG>::kEven);
+                        if (ragged && lane == 0) *(volatile int*)&Q.ragged = 1;
+                    }
+                }
+                if (inside < need || ragged || wave_exhausted(Q)) break;
             }
             if (p >= 0) {
                 if constexpr (!WaveShape<R, INTEG>::kInPool) boxes[p] = b;
@@ -487,7 +553,7 @@ __device__ __forceinline__ void wave_loop(const Src& src, unsigned long long* co
 #endif
     if (failed && lane == 0) {
         atomicExch(&Q.error, 1);
-        atomicAdd(&counters[kCounters - 1], 1ull);
+        atomicAdd(&counters[kTimeouts], 1ull);
     }
     __syncthreads();
 

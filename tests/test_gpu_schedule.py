@@ -1,0 +1,56 @@
+"""How the wavefront loop cuts its integration tasks (rt_wave.cuh), and the
+launch configuration's setters and tuner: nothing of it changes a result."""
+import numpy as np
+import pytest
+
+from paper_1012_5107_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+# Rays across the grooves at grazing elevation leave the box so far apart that
+# the FP32 loops begin to cut their tasks (wave_ragged, from some 100,000 steps
+# of uncut tasks on); the last camera keeps them together.
+@pytest.mark.parametrize("integrator", [0, 1, 2])
+@pytest.mark.parametrize("over", [
+    dict(azim_deg=90.0, elev_deg=10.0, E=32.0, cam_dist=40.0),
+    dict(azim_deg=60.0, elev_deg=12.0, E=16.0, cam_dist=24.0, A=0.02),
+    dict(azim_deg=90.0, elev_deg=10.0, E=32.0, cam_dist=40.0, A=0.06, flags=1),
+    dict(),
+])
+def test_cut_tasks_change_nothing(integrator, over):
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    p = inputs.base_scene(**{**dict(width=200, height=168, spp=4, precision=0, integrator=integrator, rtol=1e-5,
+                                    atol=1e-5, seed=9, max_steps=40000), **over})
+    out = []
+    for min_active in (0, 1, 32, 0):
+        sc = rt.Scene(p)
+        sc.set_launch(3, min_active)
+        rgb = torch.zeros(sc.shape, dtype=torch.float32, device="cuda")
+        rec = torch.zeros(200 * 168 * 4 * 80, dtype=torch.uint8, device="cuda")
+        sc.render(rgb, rec=rec)
+        st = sc.stats()
+        assert st["sched_timeouts"] == 0 and st["rays"] == 200 * 168 * 4
+        out.append((rgb.cpu().numpy(), rec.cpu().numpy(), st["steps"]))
+    for o in out[1:]:
+        assert np.array_equal(out[0][0], o[0], equal_nan=True) and np.array_equal(out[0][1], o[1]) and out[0][2] == o[2]
+
+
+@pytest.mark.parametrize("over", [
+    dict(precision=0), dict(precision=1), dict(precision=1, A=0.06), dict(precision=0, integrator=1),
+    dict(precision=1, integrator=1),
+])
+def test_set_launch_keeps_min_active(over):
+    """min_active 0 keeps the current one, also where the variant changes."""
+    pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    sc = rt.Scene(inputs.base_scene(width=16, height=16, **over))
+    first = sc.get_launch()["min_active"]
+    sc.set_launch(0, 0)
+    assert sc.get_launch()["min_active"] == first
+    sc.set_launch(3, 0)
+    assert sc.get_launch()["min_active"] == first
+    sc.set_launch(-1, 19)
+    sc.set_launch(0, 0)
+    assert sc.get_launch()["min_active"] == 19
