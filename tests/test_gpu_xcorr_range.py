@@ -128,34 +128,32 @@ def test_xcorr_tall_chunks_of_large_values(H, W, C, scale):
 
 
 def test_maps_of_two_threads_at_once():
-    """Calls whose tiles need different amounts of shared memory, alternated on two
-    threads' streams, give what they give alone."""
+    """Calls of one tile kernel whose plans need 92 KB and 13 KB of shared memory,
+    on two threads and streams, give what they give alone."""
     torch = pytest.importorskip("torch")
     import threading
 
     from paper_1012_5107_gb300 import rt
     torch.manual_seed(5)
-    sizes = [(96, 96, 3, 40, 40), (64, 48, 1, 1, 4), (200, 300, 3, 12, 40), (40, 33, 1, 40, 13)]
+    sizes = [(96, 96, 3, 64, 1), (200, 300, 1, 1, 40)]
     pairs = [(torch.rand(H, W, C, device="cuda"), torch.rand(H, W, C, device="cuda")) for H, W, C, _, _ in sizes]
     alone = [rt.xcorr_map([p], 50.0, 50.0, di, dj)[0].cpu() for p, (_, _, _, di, dj) in zip(pairs, sizes)]
     errors = []
 
-    def work(order):
+    def work(q):
         try:
             stream = torch.cuda.Stream()
-            outs = [torch.empty_like(a, device="cuda") for a in alone]
+            out = torch.empty_like(alone[q], device="cuda")
             peak = torch.empty(3, dtype=torch.float64, device="cuda")
             torch.cuda.synchronize()
-            for _ in range(150):
-                for q in order:
-                    rt.xcorr_map([pairs[q]], 50.0, 50.0, sizes[q][3], sizes[q][4], out=outs[q], peak=peak, stream=stream)
+            for _ in range(4000):
+                rt.xcorr_map([pairs[q]], 50.0, 50.0, sizes[q][3], sizes[q][4], out=out, peak=peak, stream=stream)
             stream.synchronize()
-            for a, o in zip(alone, outs):
-                assert torch.equal(a, o.cpu())
+            assert torch.equal(alone[q], out.cpu())
         except Exception as e:                           # noqa: BLE001 (reported by the test's own thread)
             errors.append(e)
 
-    threads = [threading.Thread(target=work, args=(o,)) for o in ((0, 1, 2, 3), (3, 1, 0, 2), (2, 3, 1, 0))]
+    threads = [threading.Thread(target=work, args=(q,)) for q in (0, 1)]
     for t in threads:
         t.start()
     for t in threads:
