@@ -171,8 +171,14 @@ using namespace grt;
     } while (0)
 
 struct rt_batch {
-    int n, device, precision, integrator, grid, nsm, min_active;
-    int mode;                // the integrator, with kModeSplit (batch_mode)
+    int n, device, precision, integrator, nsm, min_active;
+    // A render is one launch, or two where a scene may take either double
+    // precision step (rt_split.cuh): each scene takes the one it takes alone.
+    // Both are recorded, and which scenes a launch renders stands in the device
+    // table, so that an update needs no new recording; a launch without scenes
+    // ends at once.
+    int launches;
+    int mode[2], grid[2];    // the integrator, then with kModeSplit
     // The kernel's work list takes the scenes in slot order: slot j holds the
     // caller's scene order[j].  Cloaked scenes (rays that integrate) come
     // first, then bare gratings, then flat mirrors; within a kind the scene
@@ -182,37 +188,55 @@ struct rt_batch {
     // would.  The cheap air-only renders fill the end of the launch.
     std::vector<int> order;
     int64_t total, total_samples;
-    DevScene* d_scenes;
+    DevScene* d_scenes;      // the table: n scenes, then per launch the first sample of each scene in it (n + 1;
+                             // a scene of the other launch has none)
     int64_t* d_offsets;      // first pixel of each scene
-    int64_t* d_soffsets;     // first sample of each scene
     float* d_samp;           // per-sample colours of multi-sample pixels
     int* d_pcnt;             // per-pixel sample counters
     void* d_br;              // Fresnel branch queues (when a scene has RT_FLAG_FRESNEL)
     bool opt;                // a scene has options (RT_FLAG_*): the options build of the loop
     std::vector<DevScene> h_scenes;    // the table last uploaded
-    DevScene* h_stage;       // pinned staging of rt_batch_update
+    unsigned char* h_stage;  // pinned staging of rt_batch_update
     cudaEvent_t staged;      // the last staging copy is done
     float** d_rgbs;
     std::vector<float*> h_rgbs;        // output pointers last uploaded
     unsigned long long* d_counters;
     cudaGraph_t graph;
     cudaGraphExec_t exec;
-    int graph_min_active, graph_mode;
+    int graph_min_active;
     cudaEvent_t done;
 };
 
-// The mode a batch's launch is compiled for: the split double precision steps
-// where every cloaked scene is within their bounds (the others integrate
-// nothing).
-static int batch_mode(int precision, int integrator, bool opt, const std::vector<DevScene>& scenes)
+static size_t table_bytes(const rt_batch* b)
 {
-    bool cloaked = false;
-    for (const DevScene& s : scenes) {
-        if (!s.cloak) continue;
-        cloaked = true;
-        if (wave_mode(precision, integrator, s) == integrator) return integrator;
+    return sizeof(DevScene) * (size_t)b->n + sizeof(int64_t) * (size_t)b->launches * (size_t)(b->n + 1);
+}
+
+// The launch that renders each scene.  Scenes without a cloak integrate
+// nothing and give the same image in both: they fill the end of the second
+// where it has scenes.
+static std::vector<int> assign_launches(const rt_batch* b, const std::vector<DevScene>& scenes)
+{
+    std::vector<int> launch(scenes.size(), 0);
+    if (b->launches == 1) return launch;
+    int bare = 0;
+    for (size_t j = 0; j < scenes.size(); ++j)
+        if (scenes[j].cloak && wave_mode(b->precision, b->integrator, scenes[j]) != b->integrator) launch[j] = bare = 1;
+    for (size_t j = 0; j < scenes.size(); ++j)
+        if (!scenes[j].cloak) launch[j] = bare;
+    return launch;
+}
+
+static void fill_table(const rt_batch* b, const std::vector<DevScene>& scenes, unsigned char* out)
+{
+    const std::vector<int> launch = assign_launches(b, scenes);
+    memcpy(out, scenes.data(), sizeof(DevScene) * scenes.size());
+    int64_t* first = reinterpret_cast<int64_t*>(out + sizeof(DevScene) * scenes.size());
+    for (int l = 0; l < b->launches; ++l, first += b->n + 1) {
+        first[0] = 0;
+        for (int j = 0; j < b->n; ++j)
+            first[j + 1] = first[j] + (launch[j] == l ? scenes[j].nwork * scenes[j].spp : 0);
     }
-    return cloaked && !opt && precision == RT_FP64 ? integrator | kModeSplit : integrator;
 }
 
 extern "C" {
@@ -223,7 +247,8 @@ int rt_batch_create(rt_scene* const* scenes, int32_t n, rt_batch** out)
     *out = nullptr;
     RT_REQ(scenes && n >= 1, "need at least one scene");
     std::vector<DevScene> user(n), dev(n);
-    std::vector<int64_t> off(n + 1, 0), soff(n + 1, 0);
+    std::vector<int64_t> off(n + 1, 0);
+    int64_t samples = 0;
     int precision = -1, integrator = -1, device = -1;
     bool fresnel = false, opt = false;
     for (int i = 0; i < n; ++i) {
@@ -250,7 +275,7 @@ int rt_batch_create(rt_scene* const* scenes, int32_t n, rt_batch** out)
     for (int j = 0; j < n; ++j) {
         dev[j] = user[order[j]];
         off[j + 1] = off[j] + dev[j].nwork;
-        soff[j + 1] = soff[j] + dev[j].nwork * dev[j].spp;
+        samples += dev[j].nwork * dev[j].spp;
         dev[j].col_base = cols;
         if (dev[j].spp > 1) cols += dev[j].nwork * (col_block_bytes(dev[j].spp) >> 2);
     }
@@ -265,37 +290,41 @@ int rt_batch_create(rt_scene* const* scenes, int32_t n, rt_batch** out)
     b->precision = precision;
     b->integrator = integrator;
     b->total = off[n];
-    b->total_samples = soff[n];
-    b->mode = batch_mode(precision, integrator, opt, dev);
-    b->min_active = default_min_active(precision, b->mode);
-    b->graph_min_active = b->graph_mode = -1;
+    b->total_samples = samples;
+    b->opt = opt;
+    b->h_scenes = dev;
+    b->mode[0] = integrator;
+    b->mode[1] = integrator | kModeSplit;
+    b->launches = precision == RT_FP64 && !opt && integrator != RT_RK4T ? 2 : 1;
+    b->min_active = default_min_active(precision, integrator);
+    b->graph_min_active = -1;
     b->h_rgbs.assign(n, nullptr);
-    cudaError_t e = cudaMalloc(&b->d_scenes, sizeof(DevScene) * n);
+    std::vector<unsigned char> table(table_bytes(b));
+    fill_table(b, dev, table.data());
+    cudaError_t e = cudaMalloc(&b->d_scenes, table.size());
     if (e == cudaSuccess) e = cudaMalloc(&b->d_offsets, sizeof(int64_t) * (n + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_soffsets, sizeof(int64_t) * (n + 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_samp, sizeof(float) * (size_t)(cols > 0 ? cols : 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_pcnt, kScratchBytesPerPixel * (size_t)b->total);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_rgbs, sizeof(float*) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_counters, sizeof(unsigned long long) * kCounters);
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_scenes, dev.data(), sizeof(DevScene) * n, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(b->d_scenes, table.data(), table.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_offsets, off.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_soffsets, soff.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_rgbs, 0, sizeof(float*) * n);
     if (e == cudaSuccess) e = cudaMemset(b->d_counters, 0, sizeof(unsigned long long) * kCounters);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming);
-    int bps = 0;
-    b->opt = opt;
-    b->h_scenes = dev;
-    if (e == cudaSuccess) e = batch_occupancy(precision, b->mode, opt, &bps);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, device);
+    for (int l = 0; l < b->launches && e == cudaSuccess; ++l) {
+        int bps = 0;
+        e = batch_occupancy(precision, b->mode[l], opt, &bps);
+        b->grid[l] = (bps > 0 ? bps : 1) * b->nsm;
+    }
     if (e != cudaSuccess) {
         set_error("rt_batch_create: %s", cudaGetErrorString(e));
         rt_batch_destroy(b);
         return e == cudaErrorMemoryAllocation ? RT_ENOMEM : RT_ECUDA;
     }
-    b->grid = (bps > 0 ? bps : 1) * b->nsm;
     if (fresnel) {
-        e = cudaMalloc(&b->d_br, branch_queue_bytes(precision, integrator, b->grid));
+        e = cudaMalloc(&b->d_br, branch_queue_bytes(precision, integrator, b->grid[0]));
         if (e != cudaSuccess) {
             set_error("rt_batch_create: %s", cudaGetErrorString(e));
             rt_batch_destroy(b);
@@ -314,7 +343,6 @@ void rt_batch_destroy(rt_batch* b)
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->d_scenes) cudaFree(b->d_scenes);
     if (b->d_offsets) cudaFree(b->d_offsets);
-    if (b->d_soffsets) cudaFree(b->d_soffsets);
     if (b->d_samp) cudaFree(b->d_samp);
     if (b->d_pcnt) cudaFree(b->d_pcnt);
     if (b->d_br) cudaFree(b->d_br);
@@ -348,25 +376,18 @@ int rt_batch_update(rt_batch* b, const rt_scene_desc* descs, int32_t n, void* st
         dev[j].pix_list = nullptr;
         dev[j].col_base = old.col_base;
     }
-    const int mode = batch_mode(b->precision, b->integrator, b->opt, dev);
-    if (mode != b->mode) {                      // another kernel: its grid, and the launch recorded again
-        int bps = 0;
-        RT_CK(batch_occupancy(b->precision, mode, b->opt, &bps));
-        b->mode = mode;
-        b->grid = (bps > 0 ? bps : 1) * b->nsm;
-    }
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t bytes = sizeof(DevScene) * (size_t)n;
+    const size_t bytes = table_bytes(b);
     if (!b->h_stage) {
         RT_CK(cudaMallocHost((void**)&b->h_stage, bytes));
         RT_CK(cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming));
     } else {
         RT_CK(cudaEventSynchronize(b->staged));     // the previous copy has left the staging buffer
     }
-    memcpy(b->h_stage, dev.data(), bytes);
+    fill_table(b, dev, b->h_stage);
     RT_CK(cudaMemcpyAsync(b->d_scenes, b->h_stage, bytes, cudaMemcpyHostToDevice, st));
-    RT_CK(cudaEventRecord(b->staged, st));
     b->h_scenes = dev;
+    RT_CK(cudaEventRecord(b->staged, st));
     if (h2d_bytes) *h2d_bytes = bytes;
     return RT_OK;
 }
@@ -384,19 +405,23 @@ int rt_batch_render(rt_batch* b, float* const* d_rgb, void* stream)
         RT_CK(cudaMemcpyAsync(b->d_rgbs, b->h_rgbs.data(), sizeof(float*) * b->n, cudaMemcpyHostToDevice, st));
         RT_CK(cudaStreamSynchronize(st));
     }
-    if (!b->exec || b->graph_min_active != b->min_active || b->graph_mode != b->mode) {
+    if (!b->exec || b->graph_min_active != b->min_active) {
         if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
         if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
-        // record the launch (counter reset and the persistent kernel) once
+        // record the launches (counter reset and the persistent kernels) once
         cudaStream_t cap;
         RT_CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counters, 0, sizeof(unsigned long long) * kCounters, cap);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_pcnt, 0, kScratchBytesPerPixel * (size_t)b->total, cap);
-        const BatchLaunch L = {b->d_scenes, b->d_offsets, b->d_soffsets, b->d_rgbs, b->n, b->total,
-                               b->total_samples, {b->d_samp, b->d_pcnt, b->d_br}, b->d_counters, b->min_active,
-                               b->grid, b->opt};
-        if (e == cudaSuccess) e = launch_batch(b->precision, b->mode, L, cap);
+        for (int l = 0; l < b->launches && e == cudaSuccess; ++l) {
+            const int64_t* soffsets = reinterpret_cast<const int64_t*>(b->d_scenes + b->n) + (size_t)l * (b->n + 1);
+            const BatchLaunch L = {b->d_scenes, b->d_offsets, soffsets, b->d_rgbs, b->n, b->total,
+                                   b->total_samples, {b->d_samp, b->d_pcnt, b->d_br}, b->d_counters, b->min_active,
+                                   b->grid[l], b->opt};
+            if (l) e = cudaMemsetAsync(b->d_counters, 0, sizeof(unsigned long long), cap);   // the work counter
+            if (e == cudaSuccess) e = launch_batch(b->precision, b->mode[l], L, cap);
+        }
         cudaGraph_t g = nullptr;
         const cudaError_t e2 = cudaStreamEndCapture(cap, &g);
         cudaStreamDestroy(cap);
@@ -405,7 +430,6 @@ int rt_batch_render(rt_batch* b, float* const* d_rgb, void* stream)
         b->graph = g;
         RT_CK(cudaGraphInstantiate(&b->exec, b->graph, 0));
         b->graph_min_active = b->min_active;
-        b->graph_mode = b->mode;
     }
     RT_CK(cudaGraphLaunch(b->exec, st));
     RT_CK(cudaEventRecord(b->done, st));
@@ -439,7 +463,11 @@ int rt_batch_get_launch(rt_batch* b, int32_t* min_active, int32_t* grid, int64_t
 {
     RT_REQ(b, "batch is NULL");
     if (min_active) *min_active = b->min_active;
-    if (grid) *grid = b->grid;
+    if (grid) {
+        *grid = b->grid[0];
+        for (int l : assign_launches(b, b->h_scenes))
+            if (l) *grid = b->grid[1];
+    }
     if (total) *total = b->total;
     return RT_OK;
 }
@@ -479,7 +507,7 @@ int rt_batch_autotune(rt_batch* b, float* const* d_rgb, int32_t trials, void* st
     if (!tune_lookup(key, &v, &m)) {
         const int cand[] = {12, 16, 20, 24, 28};
         float best = 1e30f;
-        m = default_min_active(b->precision, b->mode);
+        m = b->min_active;
         for (int c : cand) {
             b->min_active = c;
             float ms = 0.0f;

@@ -157,7 +157,7 @@ namespace grt {
 bool tune_lookup(const std::string& key, int* variant, int* min_active);
 // Scene table of a validated descriptor (texture pointer left to the caller).
 void build_scene_table(const rt_scene_desc* d, DevScene* s);
-// `mode`: the integrator, with kModeSplit where every cloaked scene takes it.
+// `mode`: the integrator, with kModeSplit for the launch of the scenes that take it.
 cudaError_t batch_occupancy(int precision, int mode, bool opt, int* bps);
 // One launch of the wavefront loop over the pixels of n scenes (device tables).
 struct BatchLaunch {

@@ -602,6 +602,11 @@ __global__ void __launch_bounds__(WaveShape<R, INTEG>::kBlock, WaveShape<R, INTE
     float* const* __restrict__ rgbs, int n, int64_t total, int64_t total_samples, float* samp_col, int* pix_cnt,
     void* branches, unsigned long long* counters, int min_active)
 {
+    // (double precision: a launch holds the samples that its table says)
+    if constexpr (sizeof(R) == 8) {
+        total_samples = __ldg(soffsets + n);
+        if (total_samples == 0) return;
+    }
     const ManyScenes src{scenes, offsets, soffsets, rgbs, n, total, total_samples, samp_col, pix_cnt, branches};
     wave_loop<R, INTEG, OPT>(src, counters, min_active, WaveWait{kWaveSpin, 0});
 }
