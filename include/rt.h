@@ -267,12 +267,13 @@ int rt_scene_set_wait_limit(rt_scene* scene, int32_t spin_limit, int32_t hold_lo
 /*
  * rt_scene_autotune: time the scene's launch configurations (every
  * register-budget variant compiled for its precision and integrator, times
- * min_active in {12, 16, 20, 24, 28}; median of `trials` full renders into
- * d_rgb, which must hold one image) and keep the fastest.  The choice is
- * cached per scene class (precision, integrator, mirror, cloak and the power
- * of two of width * height * spp) for the process, and in the text file named
- * by the environment variable RT_AUTOTUNE_CACHE if set; a cached class is not
- * timed again.  Synchronous.  Outputs (nullable) report the choice.
+ * min_active in {12, 16, 20, 24, 28} and its default; median of `trials` full
+ * renders into d_rgb, which must hold one image) and keep the fastest.  The
+ * choice is cached per scene class (precision, integrator, mirror, cloak, the
+ * FP64 step the scene takes and the power of two of width * height * spp) for
+ * the process, and in the text file named by the environment variable
+ * RT_AUTOTUNE_CACHE if set; a cached class is not timed again.  Synchronous.
+ * Outputs (nullable) report the choice.
  */
 int rt_scene_autotune(rt_scene* scene, float* d_rgb, int32_t trials, void* stream, int32_t* variant,
                       int32_t* min_active);

@@ -552,14 +552,17 @@ int rt_scene_autotune(rt_scene* s, float* d_rgb, int32_t trials, void* stream, i
     RT_REQ(trials >= 1 && trials <= 64, "trials must be 1..64");
     const rt_scene_desc& d = s->desc;
     // scenes of one class share a configuration: precision, integrator,
-    // cloak and the power of two of the number of samples
+    // cloak, the wavefront loop's step (kModeSplit) and the power of two of the
+    // number of samples
     const double samples = (double)s->dev.nwork * d.spp;
+    const int mode = wave_mode(d.precision, render_mode(d), s->dev);
+    const bool split = (mode & kModeSplit) != 0;
     char key[160];
-    snprintf(key, sizeof key, "scene/p%d/i%d/c%d/m%d/f%d/log2n%d", d.precision, d.integrator, d.cloak, d.mirror, d.flags,
-             (int)floor(log2(samples > 1.0 ? samples : 1.0)));
-    int v = kDefaultVariant, m = default_min_active(d.precision, wave_mode(d.precision, render_mode(d), s->dev));
+    snprintf(key, sizeof key, "scene" RT_TUNE_GENERATION "/p%d/i%d/c%d/m%d/f%d/s%d/log2n%d", d.precision, d.integrator,
+             d.cloak, d.mirror, d.flags, split, (int)floor(log2(samples > 1.0 ? samples : 1.0)));
+    int v = kDefaultVariant, m = default_min_active(d.precision, mode);
     if (!tune_lookup(key, &v, &m)) {
-        const int cand[] = {12, 16, 20, 24, 28};
+        const int dflt = m;
         cudaStream_t st = (cudaStream_t)stream;
         cudaEvent_t e0, e1;
         RT_CK(cudaEventCreate(&e0));
@@ -569,7 +572,7 @@ int rt_scene_autotune(rt_scene* s, float* d_rgb, int32_t trials, void* stream, i
         for (int var = 0; var < kVariants && rc == RT_OK; ++var) {
             if (!variant_compiled(d.precision, render_mode(d), var)) continue;
             if (d.flags != 0 && var != kVariantWave) continue;
-            for (int c : cand) {
+            for (int c : tune_candidates(dflt, var == kVariantWave && split)) {
                 rc = rt_scene_set_launch(s, var, c);
                 if (rc != RT_OK) break;
                 rc = render_common(s, nullptr, s->dev.nwork, d_rgb, nullptr, nullptr, stream);   // warm-up

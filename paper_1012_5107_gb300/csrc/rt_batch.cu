@@ -130,6 +130,14 @@ static void tune_store_locked()
     fclose(f);
 }
 
+std::vector<int> tune_candidates(int dflt, bool only_default)
+{
+    if (only_default) return {dflt};
+    std::vector<int> c = {12, 16, 20, 24, 28};
+    if (std::find(c.begin(), c.end(), dflt) == c.end()) c.push_back(dflt);
+    return c;
+}
+
 bool tune_lookup(const std::string& key, int* variant, int* min_active)
 {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
@@ -501,14 +509,18 @@ int rt_batch_autotune(rt_batch* b, float* const* d_rgb, int32_t trials, void* st
 {
     RT_REQ(b && d_rgb, "batch and d_rgb must not be NULL");
     RT_REQ(trials >= 1 && trials <= 64, "trials must be 1..64");
+    // which of the two launches have scenes: min_active is the first's
+    const std::vector<int> launch = assign_launches(b, b->h_scenes);
+    const int second = (int)std::count(launch.begin(), launch.end(), 1);
     char key[128];
-    snprintf(key, sizeof key, "batch/p%d/i%d/n%d", b->precision, b->integrator, b->n);
+    snprintf(key, sizeof key, "batch" RT_TUNE_GENERATION "/p%d/i%d/f%d/s%d/n%d", b->precision, b->integrator, b->opt,
+             second == 0 ? 0 : second == b->n ? 1 : 2, b->n);
     int v = 0, m = 0;
     if (!tune_lookup(key, &v, &m)) {
-        const int cand[] = {12, 16, 20, 24, 28};
         float best = 1e30f;
-        m = b->min_active;
-        for (int c : cand) {
+        const int dflt = default_min_active(b->precision, b->integrator);
+        m = dflt;
+        for (int c : tune_candidates(dflt, second == b->n)) {
             b->min_active = c;
             float ms = 0.0f;
             const int rc = time_batch(b, d_rgb, (cudaStream_t)stream, trials, &ms);

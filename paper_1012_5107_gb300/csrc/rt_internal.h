@@ -153,8 +153,17 @@ void counters_to_stats(const unsigned long long* c, rt_stats* out);
 // Autotuner cache (process lifetime, optionally the RT_AUTOTUNE_CACHE file).
 }  // namespace grt
 #include <string>
+#include <vector>
 namespace grt {
 bool tune_lookup(const std::string& key, int* variant, int* min_active);
+// The min_active values to time: five, and the default where it is not one of
+// them, so that tuning cannot leave a scene slower than it was; the default
+// alone for the loops that do not heed it.
+std::vector<int> tune_candidates(int dflt, bool only_default);
+// Part of every key: choices that an earlier build's kernels were timed for
+// (RT_AUTOTUNE_CACHE keeps them across builds) are not taken over.  Counted up
+// when the loops' schedule changes.
+#define RT_TUNE_GENERATION "2"
 // Scene table of a validated descriptor (texture pointer left to the caller).
 void build_scene_table(const rt_scene_desc* d, DevScene* s);
 // `mode`: the integrator, with kModeSplit for the launch of the scenes that take it.

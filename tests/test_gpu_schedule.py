@@ -1,11 +1,16 @@
 """How the wavefront loop cuts its integration tasks (rt_wave.cuh), and the
 launch configuration's setters and tuner: nothing of it changes a result."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 from paper_1012_5107_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 # Rays across the grooves at grazing elevation leave the box so far apart that
@@ -54,3 +59,31 @@ def test_set_launch_keeps_min_active(over):
     sc.set_launch(-1, 19)
     sc.set_launch(0, 0)
     assert sc.get_launch()["min_active"] == 19
+
+
+TUNE = """
+import torch
+from paper_1012_5107_gb300 import inputs, rt
+for over in (dict(), dict(A=0.06), dict(integrator=1), dict(integrator=1, rtol=1e-4, atol=1e-4)):
+    p = inputs.base_scene(width=24, height=20, spp=1, precision=1, **over)
+    sc = rt.Scene(p)
+    print(sc.autotune(torch.zeros(sc.shape, dtype=torch.float32, device="cuda"), trials=1)["variant"])
+    b = rt.Batch([sc])
+    b.autotune([torch.zeros(sc.shape, dtype=torch.float32, device="cuda")], trials=1)
+"""
+
+
+def test_tuned_choices_are_kept_apart(tmp_path):
+    """Scenes that take different FP64 steps are tuned apart, and choices that a
+    file holds from an earlier build's kernels are left alone and not taken."""
+    pytest.importorskip("torch")
+    cache = tmp_path / "tune"
+    old = ["batch/p1/i0/n1 0 13", "batch/p1/i1/n1 0 13", "scene/p1/i0/c1/m1/f0/log2n8 0 13", "scene/p1/i1/c1/m1/f0/log2n8 0 13"]
+    cache.write_text("\n".join(old) + "\n")
+    run = subprocess.run([sys.executable, "-c", TUNE], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                         env=dict(os.environ, RT_AUTOTUNE_CACHE=str(cache)))
+    assert run.returncode == 0, run.stderr[-2000:]
+    lines = cache.read_text().split("\n")
+    new = [x for x in lines if x and x not in old]
+    assert all(x in lines for x in old) and len(new) == 8
+    assert not any(x.endswith(" 13") for x in new)
