@@ -70,8 +70,8 @@ extern "C" {
                                  step h in t; wavefront loop only              */
 #define RT_FP32 0             /* single precision bulk arithmetic              */
 #define RT_FP64 1             /* double precision throughout (rt_split.cuh:
-                                 partly as sums of two and three floats, with
-                                 no more rounding)                             */
+                                 partly as sums of two and three floats, where
+                                 they are as accurate)                         */
 
 /* per-ray status */
 #define RT_RAY_OK 0           /* reached the background                        */

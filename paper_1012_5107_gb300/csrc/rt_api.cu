@@ -276,25 +276,21 @@ static void build_dev(const rt_scene_desc* d, DevScene* s)
         s->cd.far24 = reach > 4.0 * Mth<double>::kPredTol ? 1.0 : 0.0;
     }
     // The split double precision steps (rt_split.cuh): plain grating cloaks, RK4
-    // in tau or Dormand-Prince, within the bounds their series are cut for --
-    // kA <= 0.3 and a step's |D| <= k h |p|, at most 1/16 for RK4 (the
-    // benchmark's h = Lambda/200 has 0.042 at kA = 0.25) and 0.56 for
-    // Dormand-Prince (h_max = Lambda/16: 0.53) -- and with |W0| >= kA exp(-50)
-    // in the box, where its FP32 parts keep their relative precision.
-    // Dormand-Prince at tolerances past 1e-6 takes steps so long that the
-    // carried W0's rounding shows (1.0e-15 at the end of a ray against 8.5e-16
-    // at 1e-4; none at 1e-7): the general step.
+    // in tau or Dormand-Prince, with steps within their range, of at least
+    // k h = 1e-6, and with |W0| >= kA exp(-50) in the box, where its FP32 parts keep
+    // their relative precision.  Dormand-Prince at tolerances past 1e-6 takes
+    // steps so long that the carried W0's rounding shows (1.0e-15 at the end of a
+    // ray against 8.5e-16 at 1e-4; none at 1e-7): the general step.
     {
-        const double pmax = 1.001 / (1.0 - s->kA);
         const bool rk4 = d->integrator == RT_RK4;
-        const double largest = kTwoPi * (rk4 ? s->h : std::max(s->h, s->hmax)) * pmax;
+        const bool dp45 = d->integrator == RT_DP45 && s->rtol <= 1e-6 && s->atol <= 1e-6;
         s->sp.kh = kTwoPi * s->h;
         s->sp.ikh = 1.0 / s->sp.kh;
         const double kappa = s->sp.kh * s->sp.kh * (s->cd.fk * (1.0 / kTwoPi));
         s->sp.kappa.h = (float)kappa;
         s->sp.kappa.l = (float)(kappa - (double)s->sp.kappa.h);
-        s->sp.ok = d->cloak && d->mirror == RT_MIRROR_TROCHOID && d->flags == 0 &&
-                   (rk4 || (d->integrator == RT_DP45 && s->rtol <= 1e-6 && s->atol <= 1e-6)) && s->kA <= 0.3 && largest <= (rk4 ? 1.0 / 16.0 : 0.56) &&
+        s->sp.ok = d->cloak && d->mirror == RT_MIRROR_TROCHOID && d->flags == 0 && (rk4 || dp45) &&
+                   split_in_range(rk4, s->kA, kTwoPi * (rk4 ? s->h : std::max(s->h, s->hmax))) &&
                    s->sp.kh >= 1e-6 && kTwoPi * s->ytop <= 50.0;
     }
     s->cd.ybot = ((d->flags & RT_FLAG_PLATE) || d->mirror == RT_MIRROR_GAUSS) ? 0.0 : -s->A;

@@ -25,8 +25,8 @@
 //   d + W_b (exp(d) - 1) = D.
 // d is small, so exp(d) - 1 is a short Taylor polynomial and no argument
 // reduction, library exponential or sine is needed.  The solve (split_solve)
-// takes d0 in FP32 (third-order continuation and one Newton step), then one
-// Newton step on the residual in two floats.  The abscissa itself never enters.
+// takes d0 in FP32 (fourth-order continuation), then one Newton step on the
+// residual in two floats.  The abscissa itself never enters.
 //
 // What bounds it.  846 single and some 450 packed FP32 instructions a step
 // against the FP64 step's 600 FP64 instructions of 64 scheduler cycles each.
@@ -37,14 +37,22 @@
 // evaluations with the sums on packed pairs 50 ms, the face tests out of FP64
 // and the state in shared memory 44 ms, fewer normalisations 39 ms.
 //
-// Accuracy, against RK4 of the same step in 113 bits over 1,000 rays of up to
-// 1,500 steps at kA = 0.25, h = Lambda/200: largest error of (x, y, p_x, p_y)
-// at the end of a ray 1.1e-15 median, 4.0e-15 for 90 % of the rays, 1.9e-14 for
-// 99 %; the FP64 step 2.8e-15, 1.2e-14, 4.2e-14.  (kA = 0.13: 5.9e-16 median
-// against 2.2e-15.)
-//
-// The step is used where its bounds hold (build_dev in rt_api.cu): steps of
-// |D| <= 1/16, kA <= 0.3, and W0 at the box's top far from FP32 underflow.
+// Accuracy.  Two floats are 48 bits against FP64's 53, and the solve's errors grow
+// with a high power of its |d|, so the step is no less accurate than FP64's
+// only up to some step size (split_in_range).  At that range's edge, over 100
+// rays of up to 300 steps, half of them from the crests upwards, against RK4 of
+// the same step in 113 bits: error of (x, y, p_x, p_y), median / 90 % of the rays,
+// and in parentheses of RK4 in double (tests/test_split_accuracy.py):
+//   kA = 0.02   2.3e-16 / 5.1e-16  (1.2e-15 / 2.1e-15)
+//   kA = 0.1    4.2e-16 / 1.6e-15  (1.1e-15 / 2.5e-15)
+//   kA = 0.25   1.5e-16 / 6.3e-16  (9.8e-16 / 1.8e-15)
+//   kA = 0.3    1.5e-16 / 7.9e-16  (8.8e-16 / 2.0e-15)
+// (kA = 0.3 at steps half as long again, with the guess cut at t^3: 3.5e-16 /
+// 4.8e-15, rms 11 times the double's.)  Dormand-Prince with its stages' W0 so, and
+// steps chosen for 1e-6: the double's within 7 %.  Whole rays, the kernels'
+// exits against a trace with 64-bit mantissas, 2,464 rays a scene, kA from 0.005
+// to 0.3: RK4's median error 0.1 to 0.9 of the FP64 kernel's and its rms 0.3 to
+// 1.0; Dormand-Prince's 0.98 to 1.02.
 #pragma once
 
 #if defined(__CUDACC__)
@@ -99,6 +107,21 @@ GRT_HD float2 vfma(float2 a, float2 b, float2 c) { return {ffma(a.x, b.x, c.x), 
 GRT_HD float2 vmul(float2 a, float2 b) { return {a.x * b.x, a.y * b.y}; }
 #endif
 GRT_HD float2 vneg(float2 a) { return {-a.x, -a.y}; }
+
+// Whether scenes of amplitude kA whose steps are h at most (kh = k h) take these
+// steps.  A step's displacement is D <= k h n_max, n_max = 1/(1 - kA) (a thousandth
+// for the drift of |p| over a ray), and the solve's |d| up to D/(1 - kA).
+// RK4: |d| <= 0.06, where the series of split_expm1_tail and the guess still
+// leave it no less accurate than FP64's (the benchmark's h = Lambda/200 has
+// 0.056 at kA = 0.25); up to kA = 0.1, where forces and W0 are smaller, |D| <= 1/16.
+// Dormand-Prince, whose stages' W0 alone is carried, for
+// one step, and enters scaled by it: |D| <= 0.56 (h_max = Lambda/16 has 0.53 at
+// kA = 0.25) and kA <= 0.28 (at 0.3 a tenth of the rays end up to 30 % further off).
+inline bool split_in_range(bool rk4, double kA, double kh)
+{
+    const double D = kh * (1.001 / (1.0 - kA));
+    return rk4 ? kA <= 0.3 && D <= (kA <= 0.1 ? 1.0 / 16.0 : 0.06 * (1.0 - kA)) : kA <= 0.28 && D <= 0.56;
+}
 
 struct F2 { float h, l; };          // h + l, |l| <= ulp(h)/2 when normalised
 struct Z2 { float2 h, l; };         // a pair (x, y) of those: a point, or re + i im
@@ -170,11 +193,6 @@ GRT_HD Z2 zmulu(Z2 a, Z2 b)                       // not normalised
     const float tx = ffma(-a.l.y, b.h.y, ffma(-a.h.y, b.l.y, ffma(a.l.x, b.h.x, ffma(a.h.x, b.l.x, p.l))));
     const float ty = ffma(a.l.y, b.h.x, ffma(a.h.y, b.l.x, ffma(a.l.x, b.h.y, ffma(a.h.x, b.l.y, q.l))));
     return {s.h, vadd(s.l, vadd(float2{tx, ty}, float2{u.l, v.l}))};
-}
-GRT_HD Z2 zmul(Z2 a, Z2 b)
-{
-    const Z2 s = zmulu(a, b);
-    return fast_two_sum(s.h, s.l);
 }
 GRT_HD Z2 zmulf(Z2 a, float2 b)                   // times a complex float, not normalised
 {
@@ -255,9 +273,10 @@ GRT_HD void split_force(Z2 w, F2 kappa, Z2& f, Z2& r)
     r = mul(Z2{float2{a.h, -b.h}, float2{a.l, -b.l}}, inv);
 }
 
-// exp(z) - 1 = z + e for a complex float z, |z| <= 0.06: Taylor to the ninth
-// order, z^2 (1/2 + z U), U = 1/3! + z V, V = 1/4! + z X, with X and the
-// products that enter below 2^-48 of the result in FP32.
+// exp(z) - 1 = z + e for a complex float z: Taylor to the ninth order,
+// z^2 (1/2 + z U), U = 1/3! + z V, V = 1/4! + z X, with X and the products that
+// enter below 2^-48 of the result in FP32 -- for |z| <= 0.06; at 0.13
+// (split_solve_wide) the change of W0 is off by up to 1.7e-14 of itself (rms).
 GRT_HD Z2 split_expm1_tail(float2 z)
 {
     const float c5l = -0x1.dddddep-32f;                            // 1/5! past its FP32 rounding
@@ -287,12 +306,17 @@ GRT_HD Z2 split_expm1_tail(float2 z)
 }
 
 // The continuation d of W = W_b exp(d) over s in FP32: with t = s r, v = W_b r,
-// d = t - v t^2/2 - v (1 - 3v) t^3/6, good to about t^4/50.
+// d = t - v t^2 (1/2 + (1 - 3v) t/6 + (1 - 10v + 15v^2) t^2/24), good to about
+// t^5/30.  (split_newton drops the third order of its error: cut at t^3 the guess
+// was most of the solve's error near the crests, 5.9e-15 of W0 at W_b = -0.3 and
+// |s| = 0.042 against 8.6e-16 so, for 0.4 % of the step's time.)
 GRT_HD float2 split_guess(float2 v, float2 r, float2 s)
 {
     const float2 t = cmul(s, r);
+    const float2 u = {ffma(0.625f, v.x, -5.0f / 12.0f), 0.625f * v.y};
+    const float2 g = cfma(u, v, float2{1.0f / 24.0f, 0.0f});                          // (1 - 10v + 15v^2)/24
     const float2 c = {ffma(-0.5f, v.x, 1.0f / 6.0f), -0.5f * v.y};                   // (1 - 3v)/6
-    const float2 a = cmul(v, cfma(c, t, float2{0.5f, 0.0f}));                         // v (1/2 + (1 - 3v) t/6)
+    const float2 a = cmul(v, cfma(cfma(g, t, c), t, float2{0.5f, 0.0f}));
     const float2 b = cmul(a, t);
     return cfma(float2{-b.x, -b.y}, t, t);
 }
