@@ -935,10 +935,16 @@ __device__ __forceinline__ void split_state(const Box<double>& b, double kh, F2 
     s.r = r.h;
 }
 
-// X, y, p, W0, 1/(1 + W0) and the force of b
+// X, y, p, W0, 1/(1 + W0) and the force of b.  The abscissa runs on over the
+// cells in s.t: the whole periods come off before it is rounded to FP64 (at
+// X = 32, 200 in units of 1/k, a product with 1/(2 pi) is off by 3e-15).
 __device__ __forceinline__ void box_of_split(const SplitState& s, double ikh, double fk, Box<double>& b)
 {
-    b.X = kInvTwoPi * join_y(s.t);
+    constexpr double kTwoPiLow = 2.4492935982947064e-16;              // 2 pi past its FP64 rounding
+    const double n = (double)rintf((float)kInvTwoPi * s.t.h.y);
+    const double x = fma(-n, kTwoPi, (double)s.t.h.y);
+    b.X = kInvTwoPi * (x + (((double)s.t.m.y + (double)s.t.l.y) - n * kTwoPiLow));
+    b.cx += n;
     b.y = -kInvTwoPi * join_x(s.t);
     b.px = ikh * join_y(s.q);
     b.py = -ikh * join_x(s.q);
