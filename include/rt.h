@@ -413,6 +413,15 @@ int rt_xcorr(const float* d_f, const float* d_g, int32_t height, int32_t width, 
              const double* fov_deg, int32_t n_fov, double hfov_deg, double* d_out, void* stream);
 
 /*
+ * rt_trim_scratch: give back the device memory that rt_xcorr and rt_xcorr_map
+ * keep between calls (up to 64 MiB a device, in a memory pool of the library's
+ * own; the next call allocates again, some 0.2 ms).  Destroying the last scene
+ * does the same; this is for programs that only score images.  Scratch in use
+ * stays until its call is done.  Host only, from any thread.
+ */
+int rt_trim_scratch(void);
+
+/*
  * rt_xcorr_noalloc: rt_xcorr without any device allocation, for callers that
  * cannot allocate -- hosts that give all device memory to their own pool and
  * forbid allocations behind its back, and latency-bound loops in which an

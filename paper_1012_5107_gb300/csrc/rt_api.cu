@@ -66,11 +66,13 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t stream)
     return cudaMallocFromPoolAsync(p, bytes, pool, stream);
 }
 
-void scratch_trim()
+cudaError_t scratch_trim()
 {
     std::lock_guard<std::mutex> lock(g_scratch_mutex);
+    cudaError_t e = cudaSuccess;
     for (cudaMemPool_t pool : g_scratch_pool)
-        if (pool) cudaMemPoolTrimTo(pool, 0);
+        if (pool && e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
+    return e;
 }
 
 }  // namespace grt
@@ -664,6 +666,13 @@ int rt_xcorr(const float* d_f, const float* d_g, int32_t height, int32_t width, 
     cudaError_t e2 = bytes ? cudaFreeAsync(partial, st) : cudaSuccess;
     RT_CK(e);
     RT_CK(e2);
+    return RT_OK;
+}
+
+int rt_trim_scratch(void)
+{
+    g_err[0] = 0;
+    RT_CK(scratch_trim());
     return RT_OK;
 }
 

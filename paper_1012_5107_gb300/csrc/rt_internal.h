@@ -131,7 +131,7 @@ size_t xcorr_scratch_bytes(int H, int W, int C, int n_fov);
 // call).  scratch_trim gives the kept memory back.
 constexpr size_t kScratchKeep = (size_t)64 << 20;
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t stream);
-void scratch_trim();
+cudaError_t scratch_trim();
 cudaError_t launch_xcorr(const float* f, const float* g, int H, int W, int C, const Windows& win, void* scratch,
                          double* out, cudaStream_t stream);
 

@@ -83,7 +83,7 @@ EXPORTS = ["rt_create_scene", "rt_destroy_scene", "rt_render", "rt_render_pixels
            "rt_batch_get_launch", "rt_batch_autotune", "rt_batch_update",
            "rt_validate_desc", "rt_request_bytes", "rt_server_create", "rt_server_destroy", "rt_submit", "rt_poll",
            "rt_server_stats",
-           "rt_xcorr", "rt_xcorr_noalloc", "rt_xcorr_map", "rt_eval_medium", "rt_last_error", "rt_version"]
+           "rt_xcorr", "rt_xcorr_noalloc", "rt_xcorr_map", "rt_trim_scratch", "rt_eval_medium", "rt_last_error", "rt_version"]
 
 
 def lib() -> C.CDLL:
@@ -359,6 +359,11 @@ def xcorr_map(pairs, fov_deg: float, hfov_deg: float, max_di: int, max_dj: int, 
     _check(lib().rt_xcorr_map(fp, gp, n, H, W, Cc, float(fov_deg), float(hfov_deg), int(max_di), int(max_dj),
                               _ptr(out), _ptr(peak), _stream(stream)))
     return out, peak
+
+
+def trim_scratch() -> None:
+    """Give back the device memory that xcorr and xcorr_map keep between calls (rt_trim_scratch)."""
+    _check(lib().rt_trim_scratch())
 
 
 def xcorr_noalloc(f, g, fov_deg, hfov_deg: float, out=None, stream=None):

@@ -159,3 +159,26 @@ def test_maps_of_two_threads_at_once():
     for t in threads:
         t.join()
     assert not errors, errors[0]
+
+
+def test_scratch_is_given_back():
+    """The memory that the correlation calls keep goes back on request, and the
+    next calls are as before."""
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    torch.manual_seed(6)
+    f, g = torch.rand(600, 640, 3, device="cuda"), torch.rand(600, 640, 3, device="cuda")
+    out, peak = rt.xcorr_map([(f, g)], 50.0, 50.0, 20, 20)
+    first = out.clone()
+    torch.cuda.synchronize()
+    rt.trim_scratch()
+    free = torch.cuda.mem_get_info()[0]
+    rt.xcorr_map([(f, g)], 50.0, 50.0, 20, 20, out=out, peak=peak)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] > 1 << 20            # some 10 MB are kept
+    rt.trim_scratch()
+    assert free - torch.cuda.mem_get_info()[0] < 1 << 20
+    rt.xcorr_map([(f, g)], 50.0, 50.0, 20, 20, out=out, peak=peak)
+    rt.trim_scratch()                                               # with the call in flight
+    torch.cuda.synchronize()
+    assert torch.equal(out, first)
