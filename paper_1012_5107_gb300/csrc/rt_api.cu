@@ -295,6 +295,18 @@ static void build_dev(const rt_scene_desc* d, DevScene* s)
                    split_in_range(rk4, s->kA, kTwoPi * (rk4 ? s->h : std::max(s->h, s->hmax))) &&
                    s->sp.kh >= 1e-6 && kTwoPi * s->ytop <= 50.0;
     }
+    // Whether the view makes neighbouring rays leave the box far apart: its centre
+    // ray crosses many grooves on its way down and up through the box, or the box
+    // is long.  RK4 at 900 x 900 x 4, uncut tasks against cut ones (rt_wave.cuh):
+    // faster up to 4.6 periods across (0.83 to 1.00 of the time), slower from 5.6
+    // (1.05 to 1.6); Dormand-Prince, with a third of the steps between services,
+    // up to 8 and from 15.
+    {
+        const double el = d->elev_deg * kPi / 180.0, az = d->azim_deg * kPi / 180.0;
+        const double along = std::min(2.0 * s->E2, 2.0 * s->H * fabs(cos(el)) / std::max(fabs(sin(el)), 1e-9));
+        const double across = along * fabs(sin(az));
+        s->ragged = d->integrator == RT_DP45 ? across >= 12.0 : across >= 5.5 || along >= 20.0;
+    }
     s->cd.ybot = ((d->flags & RT_FLAG_PLATE) || d->mirror == RT_MIRROR_GAUSS) ? 0.0 : -s->A;
     s->cf.ybot = (float)s->cd.ybot;
     // Gaussian bump: width, 1/width, k h, h/width, the Newton stop on W and

@@ -239,6 +239,14 @@ static void fill_table(const rt_batch* b, const std::vector<DevScene>& scenes, u
 {
     const std::vector<int> launch = assign_launches(b, scenes);
     memcpy(out, scenes.data(), sizeof(DevScene) * scenes.size());
+    // cut tasks for all scenes or for none (rt_wave.cuh)
+    int64_t cloaked = 0, ragged = 0;
+    for (const DevScene& s : scenes) {
+        if (!s.cloak) continue;
+        cloaked += s.nwork * s.spp;
+        if (s.ragged) ragged += s.nwork * s.spp;
+    }
+    for (int j = 0; j < b->n; ++j) reinterpret_cast<DevScene*>(out)[j].ragged = ragged > 0 && 2 * ragged >= cloaked;
     int64_t* first = reinterpret_cast<int64_t*>(out + sizeof(DevScene) * scenes.size());
     for (int l = 0; l < b->launches; ++l, first += b->n + 1) {
         first[0] = 0;

@@ -91,6 +91,8 @@ struct DevScene {
     double idx_scale;                       // index scale inside the cloak (1 + kA when referenced)
     double plate_n;                         // index of the dielectric plate (1 + kA)
     SplitConst sp;
+    int ragged;                             // neighbouring rays leave the box far apart (build_dev); in a table of
+                                            // scenes: the launch's tasks are cut (rt_wave.cuh)
 };
 
 // ------------------------------------------------------------------------

@@ -505,6 +505,7 @@ static cudaError_t publish(rt_server* S, Ring& g, Request& r)
     RingSlot& h = g.h_slot_stage[s];
     memset(&h, 0, sizeof h);
     build_scene_table(&r.desc, &h.sc);
+    h.sc.ragged = 0;                     // requests of all views share the launch (rt_wave.cuh)
     const long long npix = (long long)h.sc.nwork;
     const long long ns = npix * h.sc.spp;
     char* base = S->arena.base + r.arena_off;

@@ -42,6 +42,35 @@ def test_cut_tasks_change_nothing(integrator, over):
         assert np.array_equal(out[0][0], o[0], equal_nan=True) and np.array_equal(out[0][1], o[1]) and out[0][2] == o[2]
 
 
+@pytest.mark.parametrize("integrator", [0, 1, 2])
+def test_batches_of_either_schedule(integrator):
+    """A scene's image is the same in a batch most of whose scenes look across the
+    grooves (cut tasks) and in one of scenes that do not (uncut), and after an
+    update from the one to the other."""
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+
+    def scene(q, az):
+        return inputs.base_scene(width=112, height=80, spp=4, precision=0, integrator=integrator, rtol=1e-5, atol=1e-5,
+                                 seed=q, E=32.0, cam_dist=40.0, elev_deg=14.0, azim_deg=az)
+
+    across = [scene(q, az) for q, az in enumerate((90.0, 80.0, 75.0))]
+    along = [scene(10 + q, az) for q, az in enumerate((0.0, 4.0, -7.0))]
+    sets = {"cut": across + along[:1], "uncut": across[:1] + along, "cut again": across + along[:1]}
+    scenes = [rt.Scene(p) for p in sets["cut"]]
+    b = rt.Batch(scenes)
+    out = {}
+    for name, ps in sets.items():
+        b.update(ps)
+        img = [torch.zeros(sc.shape, dtype=torch.float32, device="cuda") for sc in scenes]
+        b.render(img)
+        assert b.stats()["sched_timeouts"] == 0
+        out[name] = img
+    b.close()
+    assert torch.equal(out["cut"][0], out["uncut"][0]) and torch.equal(out["cut"][3], out["uncut"][1])
+    assert all(torch.equal(x, y) for x, y in zip(out["cut"], out["cut again"]))
+
+
 @pytest.mark.parametrize("over", [
     dict(precision=0), dict(precision=1), dict(precision=1, A=0.06), dict(precision=0, integrator=1),
     dict(precision=1, integrator=1),
