@@ -53,9 +53,9 @@ FLOP_PER_STEP = 105
 MUFU_PER_NEWTON = 4
 # DRAM bytes (read + write) of one batched render launch of the step (the six
 # renders): dram__bytes_read.sum + dram__bytes_write.sum of an ncu capture
-# (--set full, one launch) of the current kernel; None until that capture
-# exists or after the kernel changes.
-TRAFFIC_BATCH_BYTES = None
+# (one launch) of the current kernel; None until that capture exists or after
+# the kernel changes.
+TRAFFIC_BATCH_BYTES = 5203200 + 2934016
 
 
 def peaks():

@@ -28,11 +28,11 @@
 // takes d0 in FP32 (fourth-order continuation), then one Newton step on the
 // residual in two floats.  The abscissa itself never enters.
 //
-// What bounds it.  846 single and some 450 packed FP32 instructions a step
+// What bounds it.  some 870 single and 450 packed FP32 instructions a step
 // against the FP64 step's 600 FP64 instructions of 64 scheduler cycles each.
-// The cloaked 512 x 512 x 4 render takes 39.2 ms (592 ms with the FP64 step),
+// The cloaked 512 x 512 x 4 render takes 38.0 ms (592 ms with the FP64 step),
 // the FMA pipe 65 % busy; 64 x 64 x 1, bound by the latency of the longest ray's
-// chain of steps, 5.9 ms (32.9).  On the way: unrolled 89 ms (a 2,700-instruction
+// chain of steps, 5.8 ms (32.9).  On the way: unrolled 89 ms (a 2,700-instruction
 // loop body, most issue slots waiting for instructions), rolled over the four
 // evaluations with the sums on packed pairs 50 ms, the face tests out of FP64
 // and the state in shared memory 44 ms, fewer normalisations 39 ms.

@@ -68,7 +68,7 @@ namespace grt {
 // 7.90 / 6.02, the split FP64 render 39.1 / 37.8; uncut to the very end 64 x 64 x 1
 // takes 1.52 ms instead of 1.25.  Over 128 scenes (elevations 10 to 55, azimuths
 // 0 to 90 degrees, E = 8 and 32, kA = 0.1 and 0.25, RK4 and Dormand-Prince) it is
-// within 4 % of the better of the two at 900 x 900 x 4, and within 16 % at
+// within 5 % of the better of the two at 900 x 900 x 4, and within 16 % at
 // 320 x 320 x 4, where half of the render is over before the tally tells.
 // The general FP64 builds, bound by the FP64 pipe, whose instructions cost the
 // same for few lanes as for all, are cut throughout.
@@ -81,9 +81,9 @@ constexpr int kWaveSpin = kDefaultWaitSpin;  // attempts (with a short sleep) be
 // block's lanes, so that a warp always finds work while the other warps hold
 // theirs.  FP32: two blocks of 256 threads, 128 registers.  FP32
 // Dormand-Prince keeps the running sums of its stages and two states live
-// through a step, which spills 370 bytes at 128 registers; with the step's
-// start left in the pool (kInPool: it is read at the step's ends only) it
-// spills 290 and 16 warps an SM beat the 12 that 168 registers allow (1920 x
+// through a step and spills at 128 registers; with the step's start left in
+// the pool (kInPool: it is read at the step's ends only) it spills 388 bytes (300
+// before the loop in stretches) and 16 warps an SM beat the 12 that 168 registers allow (1920 x
 // 1080 x 16, E = 2 / 8 / 32: 18.4 / 113.7 / 202.0 ms against 20.2 / 115.7 /
 // 204.0 with one block of 384; with the start in registers 19.4 / 125.2 /
 // 230.6).  FP32 RK4 in the pool is slower (7.07 -> 8.57 ms the step's launch:
@@ -255,8 +255,10 @@ __device__ __forceinline__ bool wave_exhausted(const WaveCtl& Q)
 // still inside, and says whether such tasks kept fewer than kEven percent of
 // their lanes inside of late, over all blocks of the launch.  The tally (steps,
 // and lanes / 32, in halves of a word) is halved when it reaches kTallySteps,
-// about a task's length of every warp, so it follows the work; a launch's first
-// tasks, whose early steps have all lanes inside, do not weigh on it for long.
+// about a hundred steps of every warp of the GPU, so it follows the work; a
+// launch's first tasks, whose early steps have all lanes inside, do not weigh on
+// it for long.  (Told over the whole launch it came late in small renders and, at
+// thresholds of 85 to 88 %, cut even ones: E = 8 at 55 degrees 17.8 -> 19.4 ms.)
 constexpr unsigned kTallySteps = 1u << 19;
 __device__ __forceinline__ bool wave_ragged(unsigned long long* counters, unsigned its, unsigned lanes, int even)
 {
