@@ -383,6 +383,7 @@ struct Ring {
     std::vector<uint64_t> slot_ticket;           // ticket in each slot (0: free)
     uint64_t nreq = 0;
     unsigned long long published = 0;
+    double cloaked = 0.0, ragged = 0.0;          // samples published of late: in the cloak, and of ragged views
     int grid = 0;
     bool timed_out = false;                      // a launch gave up bounded waits
 };
@@ -505,9 +506,15 @@ static cudaError_t publish(rt_server* S, Ring& g, Request& r)
     RingSlot& h = g.h_slot_stage[s];
     memset(&h, 0, sizeof h);
     build_scene_table(&r.desc, &h.sc);
-    h.sc.ragged = 0;                     // requests of all views share the launch (rt_wave.cuh)
     const long long npix = (long long)h.sc.nwork;
     const long long ns = npix * h.sc.spp;
+    // requests of all views share the launch: its tasks are cut where most of the
+    // samples published of late look across the grooves (rt_wave.cuh)
+    if (h.sc.cloak) {
+        g.cloaked = 0.75 * g.cloaked + (double)ns;
+        g.ragged = 0.75 * g.ragged + (h.sc.ragged ? (double)ns : 0.0);
+    }
+    h.sc.ragged = g.ragged > 0.0 && 2.0 * g.ragged >= g.cloaked;
     char* base = S->arena.base + r.arena_off;
     size_t at = 0;
     cudaError_t e = cudaSuccess;

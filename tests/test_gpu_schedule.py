@@ -71,6 +71,28 @@ def test_batches_of_either_schedule(integrator):
     assert all(torch.equal(x, y) for x, y in zip(out["cut"], out["cut again"]))
 
 
+def test_served_views_across_the_grooves():
+    """Requests that look across the grooves, then along them, then across again:
+    the images of the scenes alone."""
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    ps = [inputs.base_scene(width=120 + q, height=88, spp=4, precision=0, seed=30 + q, azim_deg=az)
+          for q, az in enumerate((90.0, 85.0, 78.0, 0.0, 3.0, 1.0, 88.0, 90.0))]
+    s = rt.Server(1 << 28, max_inflight=2)
+    out = [torch.zeros((p["height"], p["width"], 3), dtype=torch.float32, device="cuda") for p in ps]
+    tickets = [s.submit(p, t) for p, t in zip(ps, out)]
+    for t in tickets:
+        while s.poll(t, 1_000_000) is None:
+            pass
+    s.close()
+    for p, t in zip(ps, out):
+        sc = rt.Scene(p)
+        ref = torch.zeros_like(t)
+        sc.render(ref)
+        torch.cuda.synchronize()
+        assert torch.equal(t, ref)
+
+
 @pytest.mark.parametrize("over", [
     dict(precision=0), dict(precision=1), dict(precision=1, A=0.06), dict(precision=0, integrator=1),
     dict(precision=1, integrator=1),
