@@ -355,6 +355,7 @@ struct Request {
     int status;                        // RT_PENDING until done
     uint64_t rays;
     int passed = 0;                    // later requests admitted before it (kMaxPassed)
+    bool even = false;                 // cloaked, and of a view that is not DevScene::ragged
 };
 
 // Admission takes queued requests in arrival order, but a request that fits
@@ -383,7 +384,6 @@ struct Ring {
     std::vector<uint64_t> slot_ticket;           // ticket in each slot (0: free)
     uint64_t nreq = 0;
     unsigned long long published = 0;
-    double cloaked = 0.0, ragged = 0.0;          // samples published of late: in the cloak, and of ragged views
     int grid = 0;
     bool timed_out = false;                      // a launch gave up bounded waits
 };
@@ -508,13 +508,12 @@ static cudaError_t publish(rt_server* S, Ring& g, Request& r)
     build_scene_table(&r.desc, &h.sc);
     const long long npix = (long long)h.sc.nwork;
     const long long ns = npix * h.sc.spp;
-    // requests of all views share the launch: its tasks are cut where most of the
-    // samples published of late look across the grooves (rt_wave.cuh)
-    if (h.sc.cloak) {
-        g.cloaked = 0.75 * g.cloaked + (double)ns;
-        g.ragged = 0.75 * g.ragged + (h.sc.ragged ? (double)ns : 0.0);
-    }
-    h.sc.ragged = g.ragged > 0.0 && 2.0 * g.ragged >= g.cloaked;
+    // requests of all views share the launch: tasks are cut for one that looks
+    // across the grooves (rt_wave.cuh) where all in flight do
+    r.even = h.sc.cloak && !h.sc.ragged;
+    bool even = r.even;
+    for (int q = 0; q < kRingSlots && !even; ++q) even = g.slot_ticket[q] != 0 && S->req[g.slot_ticket[q]].even;
+    h.sc.ragged = h.sc.ragged && !even;
     char* base = S->arena.base + r.arena_off;
     size_t at = 0;
     cudaError_t e = cudaSuccess;
