@@ -355,7 +355,7 @@ struct Request {
     int status;                        // RT_PENDING until done
     uint64_t rays;
     int passed = 0;                    // later requests admitted before it (kMaxPassed)
-    bool even = false;                 // cloaked, and of a view that is not DevScene::ragged
+    bool even = false;                 // cloaked, and its view lets tasks run uncut
 };
 
 // Admission takes queued requests in arrival order, but a request that fits
@@ -508,8 +508,17 @@ static cudaError_t publish(rt_server* S, Ring& g, Request& r)
     build_scene_table(&r.desc, &h.sc);
     const long long npix = (long long)h.sc.nwork;
     const long long ns = npix * h.sc.spp;
-    // requests of all views share the launch: tasks are cut for one that looks
-    // across the grooves (rt_wave.cuh) where all in flight do
+    // Requests of all views share the launch, and cut tasks beside uncut ones are
+    // slower than either: tasks are cut (rt_wave.cuh) for a request that looks
+    // across the grooves of a long box where all in flight do.  3 requests of one
+    // view (768 x 768 x 4, elevations 8 to 20 degrees), cut against uncut, by the
+    // box's length across the view's grooves: 6 to 8 periods 0.91 to 0.97 of the
+    // time, 10 0.86 to 0.92, 12 0.78 to 0.91, 16 0.71 to 0.88, 24 0.63 to 0.72, 32
+    // 0.59 to 0.67.  200 requests of all views of a box of 8 periods: 161.0 Mrays/s
+    // with none cut, 161.8 with DevScene::ragged alone to tell, but at 80 % load
+    // mean latency 145 ms and 164.
+    const double box = 2.0 * h.sc.E2 * fabs(sin(r.desc.azim_deg * (kPi / 180.0)));
+    h.sc.ragged = h.sc.ragged && box >= 10.0;
     r.even = h.sc.cloak && !h.sc.ragged;
     bool even = r.even;
     for (int q = 0; q < kRingSlots && !even; ++q) even = g.slot_ticket[q] != 0 && S->req[g.slot_ticket[q]].even;

@@ -57,9 +57,8 @@ namespace grt {
 // that look across the grooves): all are cut if at least half of the samples
 // look so (DevScene::ragged; 8 scenes of the view above at 512 x 512 x 4: 70.8 ms
 // cut, 128 uncut), and none if not.  A served request's are cut if it and all in
-// flight with it look so (8 such requests 72.5 ms, uncut 129; 200 requests of all
-// views 161.8 Mrays/s, with none cut 161.2, with the views of most samples
-// published of late deciding 150.2).
+// flight with it look so through a long box (rt_server.cu; 8 requests of that view
+// 72.5 ms, uncut 129).
 // Below 85 % of the lanes inside an uncut RK4 render is the slower one, above
 // 89 % the faster (Dormand-Prince, with a third of the steps between services:
 // 75 and 80 %).  The options build keeps its tasks uncut (Fresnel renders at

@@ -93,6 +93,31 @@ def test_served_views_across_the_grooves():
         assert torch.equal(t, ref)
 
 
+@pytest.mark.parametrize("over", [dict(E=12.0, elev_deg=20.0), dict(E=32.0, elev_deg=10.0, cam_dist=40.0),
+                                  dict(E=32.0, elev_deg=8.0, cam_dist=40.0, integrator=1)])
+def test_served_across_a_long_box(over):
+    """Requests across the grooves of a long box, in flight by themselves (tasks
+    are cut) and beside one along them (tasks run uncut): the same images."""
+    torch = pytest.importorskip("torch")
+    from paper_1012_5107_gb300 import rt
+    ps = [inputs.base_scene(width=100 + q, height=72, spp=3, precision=0, seed=50 + q, azim_deg=90.0 - 4 * q, **over)
+          for q in range(3)]
+    along = inputs.base_scene(width=256, height=256, spp=16, precision=0, seed=60, azim_deg=0.0)
+    got = []
+    for first in ([], [along]):
+        s = rt.Server(1 << 28, max_inflight=2)
+        out = [torch.zeros((p["height"], p["width"], 3), dtype=torch.float32, device="cuda") for p in first + ps]
+        tickets = [s.submit(p, t) for p, t in zip(first + ps, out)]
+        for t in tickets:
+            while s.poll(t, 1_000_000) is None:
+                pass
+        s.close()
+        got.append(out[len(first):])
+    for a, b in zip(*got):
+        assert float(a.abs().sum()) > 0.0
+        assert torch.equal(a, b)
+
+
 @pytest.mark.parametrize("over", [
     dict(precision=0), dict(precision=1), dict(precision=1, A=0.06), dict(precision=0, integrator=1),
     dict(precision=1, integrator=1),
